@@ -851,7 +851,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1) k_acc_draw(AcceptParams p)
 #pragma unroll
                     for (int h = 0; h < 2; ++h) { tc[q][h] = tw[q][h]; sc[q][h] = sw[q][h]; }
                 fetch(vb + DW_ROWS);
-                if (!mbar_wait(&sh.full[st], (uint32_t)((n / DW_STAGES) & 1), abort)) { ok = false; break; }
+                if (!mbar_wait_warp(&sh.full[st], (uint32_t)((n / DW_STAGES) & 1), abort)) { ok = false; break; }
                 uint4 w[RANK / 32];
                 const uint8_t *src = ring + st * DW_BLOCK + (8 * warp + g) * (RANK * 2) + 16 * tq;
                 if (vb < v1) {

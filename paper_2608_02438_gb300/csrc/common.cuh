@@ -688,6 +688,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     }
 }
 
+// The same for a whole warp whose next steps are warp-collective: every lane has
+// waited, or the warp unwinds (a lane's own wait may run out, or see the abort,
+// while its neighbours' succeed).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort,
+                                               unsigned long long limit_ns = 2000000000ull)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, limit_ns));
+}
+
 __device__ __forceinline__ void fence_barrier_init()
 {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");

@@ -210,7 +210,7 @@ __device__ __forceinline__ void lm_head_body(const CUtensorMap &tmap_w, const CU
                 best[ew * NT + g * 32 + lane] = make_float2(-INFINITY, __int_as_float(0x7fffffff));
             for (int it = wk.first; it < NI && got; it += wk.step, ++t) {
                 const int buf = t % Sh::NBUF;
-                got = mbar_wait(&sh.tfull[buf], (t / Sh::NBUF) & 1, abort);
+                got = mbar_wait_warp(&sh.tfull[buf], (t / Sh::NBUF) & 1, abort);
                 tc_fence_after();
                 const int row0 = (it * MT + m) * LM_BM + q * 32, row = row0 + lane;   // this thread's vocabulary row
 #pragma unroll 1

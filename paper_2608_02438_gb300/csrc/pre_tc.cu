@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(320, 1)
         // rows 128 h .. +127 of the tile
         const int q = warp & 3, half = (warp - 2) >> 2;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        const bool got = mbar_wait(&sh.tfull, 0, abort);
+        const bool got = mbar_wait_warp(&sh.tfull, 0, abort);
         if (got) {
             tc_fence_after();
             const int t = t0 + q * 32 + lane;

@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             if (g_count == 0)
                 for (int vt = vt0; vt < vt1; ++vt) {
                     const int buf = t & 1;
-                    if (!mbar_wait(&sh.tfull[buf], (t >> 1) & 1, abort)) { ok = false; break; }
+                    if (!mbar_wait_warp(&sh.tfull[buf], (t >> 1) & 1, abort)) { ok = false; break; }
                     tc_fence_after();
                     tc_fence_before();
                     __syncwarp();
@@ -333,8 +333,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 if (gl == g_first) {
                     if (any_smp)
                         group_noise2(seed, (uint32_t)(vt * (TC_BN / GROUP) + g_first) & ~1u, (uint32_t)pos, offset, gn0, gn1);
-                    // every lane goes on, or none: what follows is for the whole warp
-                    if (!__all_sync(0xffffffffu, mbar_wait(&sh.tfull[buf], (t >> 1) & 1, abort))) { ok = false; break; }
+                    if (!mbar_wait_warp(&sh.tfull[buf], (t >> 1) & 1, abort)) { ok = false; break; }
                     tc_fence_after();
                 }
                 __syncwarp();                           // every lane has read the slot of item it - 1

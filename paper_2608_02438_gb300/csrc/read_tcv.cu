@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(TV_THREADS, 1)
             const int buf = i % TV_NBUF;
             const int v0 = (vb0 + i) * TV_BM + q * 32;          // this warp's group
             if (i + 2 < blocks) load_s_group(nxt, srow, (vb0 + i + 2) * TV_BM + q * 32, V, tvalid);
-            if (!mbar_wait(&sh.tfull[buf], (i / TV_NBUF) & 1, abort)) { ok = false; break; }
+            if (!mbar_wait_warp(&sh.tfull[buf], (i / TV_NBUF) & 1, abort)) { ok = false; break; }
             tc_fence_after();
             float acc[TV_BN];
             tmem_ld32(tmem + lane_base + buf * TV_BN, acc);     // lane: vocabulary row, acc[t]: token t

@@ -277,7 +277,7 @@ __device__ __forceinline__ void pc_consume(const Params &p, uint8_t *ring, RsSha
         for (int nt = 0; nt < NT / 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.0f;
         for (int kc = 0; kc < nchk; ++kc, ++ci) {
             const int buf = ci % Sh::BUFS;
-            if (ok && !mbar_wait(&sh.pfull[buf], (uint32_t)((ci / Sh::BUFS) & 1), abort)) ok = false;
+            if (ok && !mbar_wait_warp(&sh.pfull[buf], (uint32_t)((ci / Sh::BUFS) & 1), abort)) ok = false;
             if (ok) {
                 if (tm && kc == 0) trace_mark(p.trace, 5, t_start);
                 const int kl = min(PC_KC, H - kc * PC_KC);
@@ -591,7 +591,7 @@ __device__ __forceinline__ void read_role(const Params &p, const CUtensorMap *tm
         for (int pass = 0;; ++pass) {
             // every epilogue thread takes the same decision (the named
             // barriers below need all 256)
-            const bool got = mbar_wait(&sh.go, (uint32_t)(pass & 1), abort);
+            const bool got = mbar_wait_warp(&sh.go, (uint32_t)(pass & 1), abort);
             if (tv_epi_bar_or(!got || *abort || *reinterpret_cast<volatile int *>(&sh.pass_stop))) break;
             const unsigned long long t_go = globaltimer_ns();
             const int n = *reinterpret_cast<volatile int *>(&sh.pass_n);
@@ -628,7 +628,7 @@ __device__ __forceinline__ void read_role(const Params &p, const CUtensorMap *tm
                 const int ib = pass * nblk + i, buf = ib % TV_NBUF;
                 const int v0 = R0 + i * TV_BM + q * 32;
                 if (i + 2 < nblk) load_s_group(nxt, srow, R0 + (i + 2) * TV_BM + q * 32, V, tvalid);
-                if (!mbar_wait(&sh.tfull[buf], (uint32_t)((ib / TV_NBUF) & 1), abort)) { ok = false; break; }
+                if (!mbar_wait_warp(&sh.tfull[buf], (uint32_t)((ib / TV_NBUF) & 1), abort)) { ok = false; break; }
                 tc_fence_after();
                 float acc[TV_BN];
                 tmem_ld32(tmem + lane_base + buf * TV_BN, acc);

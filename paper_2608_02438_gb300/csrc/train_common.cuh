@@ -33,6 +33,13 @@ __device__ __forceinline__ bool mbar_wait_spin(uint64_t *bar, uint32_t parity, v
     }
 }
 
+// The same for a whole warp: every lane has waited, or the warp unwinds.
+__device__ __forceinline__ bool mbar_wait_spin_warp(uint64_t *bar, uint32_t parity, volatile int *abort,
+                                                    unsigned long long limit_ns = 2000000000ull)
+{
+    return __all_sync(0xffffffffu, mbar_wait_spin(bar, parity, abort, limit_ns));
+}
+
 // L2 prefetch of the box at (x, y) of a tiled tensor map (no shared memory,
 // no completion): a later TMA load of the same box then hits L2.
 __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *map, int x, int y)

@@ -132,7 +132,7 @@ __device__ __forceinline__ void gemm_body(const GemmArgs &g, const CUtensorMap &
 #pragma unroll
             for (int e = 0; e < (RESID ? G_BN / 4 : 0); ++e) rv[e] = *reinterpret_cast<const float4 *>(rrow + 4 * e);
         }
-        if (mbar_wait_spin(&sh.tfull, 0, abort)) {
+        if (mbar_wait_spin_warp(&sh.tfull, 0, abort)) {
             tc_fence_after();
             const bool valid = m < g.M && !*abort;
 #pragma unroll (RESID ? G_BN / 32 : 1)

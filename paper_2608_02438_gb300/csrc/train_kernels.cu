@@ -143,8 +143,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) k_train_rows(TrainMisc m)
         int k = 0;
         for (int it = blockIdx.x; it < items; it += gridDim.x, ++k) {
             const int st = k % ROWS_STAGES;
-            const bool got = mbar_wait(&sh.full[st], (uint32_t)((k / ROWS_STAGES) & 1), abort);
-            if (!__all_sync(0xffffffffu, got)) break;
+            if (!mbar_wait_warp(&sh.full[st], (uint32_t)((k / ROWS_STAGES) & 1), abort)) break;
             const int ch = it % m.nch, v0 = ch * TRAIN_ROW_CHUNK, n = min(TRAIN_ROW_CHUNK, m.V - v0);
             const uint4 *ss = reinterpret_cast<const uint4 *>(base + st * 2 * ROWS_SEG);
             const uint4 *tt = ss + ROWS_SEG / 16;
@@ -238,8 +237,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 1) k_train_rows(TrainMisc m)
         int k = 0;
         for (int it = blockIdx.x; it < items; it += gridDim.x, ++k) {
             const int pb = k % ROWS_PART;
-            const bool got = mbar_wait(&sh.pfull[pb], (uint32_t)((k / ROWS_PART) & 1), abort);
-            if (!__all_sync(0xffffffffu, got)) break;
+            if (!mbar_wait_warp(&sh.pfull[pb], (uint32_t)((k / ROWS_PART) & 1), abort)) break;
             float4 a = make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
             float b = -INFINITY;
             int bi = 0x7fffffff;

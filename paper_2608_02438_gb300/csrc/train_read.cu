@@ -417,8 +417,8 @@ __device__ __forceinline__ void train_tok_body(const TrainParams &p, const CUten
             const int buf = it % NBUF;
             const uint32_t ph = (uint32_t)((it >> 1) & 1);      // phase of the dl tile `set`
             const int ss = it % NS;
-            if (!mbar_wait_spin(&sh.tfull[buf], (uint32_t)((it / NBUF) & 1), abort, lim) ||
-                !mbar_wait_spin(&sh.sfull[ss], (uint32_t)((it / NS) & 1), abort, lim)) {
+            if (!mbar_wait_spin_warp(&sh.tfull[buf], (uint32_t)((it / NBUF) & 1), abort, lim) ||
+                !mbar_wait_spin_warp(&sh.sfull[ss], (uint32_t)((it / NS) & 1), abort, lim)) {
                 ok = false;
                 break;
             }
@@ -566,7 +566,7 @@ __device__ __forceinline__ void train_tok_body(const TrainParams &p, const CUten
                 mbar_arrive(&sh.sempty[ss]);
             }
             if (dzm) {
-                if (!mbar_wait_spin(&sh.dempty[set], ph ^ 1, abort, lim)) { ok = false; break; }
+                if (!mbar_wait_spin_warp(&sh.dempty[set], ph ^ 1, abort, lim)) { ok = false; break; }
                 uint8_t *dt = sD + set * TR_D_BUF + row * 128;
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
@@ -601,7 +601,7 @@ __device__ __forceinline__ void train_tok_body(const TrainParams &p, const CUten
                 p.part[(size_t)sv * p.NR + rowg] = a;
             }
         } else if (ok && items > 0) {
-            if (mbar_wait_spin(&sh.zdone, 0, abort, lim)) {
+            if (mbar_wait_spin_warp(&sh.zdone, 0, abort, lim)) {
                 tc_fence_after();
                 // the 4 warps of a lane quarter take 64 of the 256 columns each
                 const int c0 = (2 * set + g) * 64;
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1)
         int lt = 0, piece = 0;
         for (int vt = blockIdx.x; vt < nvt; vt += gridDim.x, ++lt) {
             const int buf = lt & 1, y = vt * DW_BM + q * 32;
-            if (!mbar_wait_spin(&sh.tfull[buf], (uint32_t)((lt >> 1) & 1), abort, lim)) break;
+            if (!mbar_wait_spin_warp(&sh.tfull[buf], (uint32_t)((lt >> 1) & 1), abort, lim)) break;
             tc_fence_after();
 #pragma unroll 1
             for (int c = 0; c < RANK / 32; ++c, ++piece) {

@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll
             for (int c = 0; c < TT_BN / 4; ++c) cv[c] = cr[c];
         }
-        const bool got = mbar_wait(&sh.tfull, 0, abort);
+        const bool got = mbar_wait_warp(&sh.tfull, 0, abort);
         if (got) {
             tc_fence_after();
             float *zf = p.z_final ? p.z_final : p.zbuf;
