@@ -660,22 +660,6 @@ struct DrawShared {
 constexpr size_t DW_SMEM = 128 + DW_STAGES * DW_BLOCK + sizeof(DrawShared);
 static_assert(DW_SMEM <= 232448, "k_acc_draw shared memory");
 
-// Barrier over the drawing warps that ORs a predicate (every one of them
-// takes the same decision to stop).
-__device__ __forceinline__ bool draw_bar_or(bool pred)
-{
-    uint32_t res;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, %2, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(res)
-        : "r"((uint32_t)pred), "n"(DW_WARPS * 32)
-        : "memory");
-    return res != 0;
-}
-
 // The bf16 values of ids v and v + 1 (v even) of a row, as one word.
 __device__ __forceinline__ uint32_t ld_pair(const void *base, size_t i, bool aligned4)
 {
@@ -796,7 +780,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1) k_acc_draw(AcceptParams p)
         int n = 0;
         for (int g0 = 0; g0 < nd; g0 += DW_NZ) {
             const int nz = min(DW_NZ, nd - g0);
-            draw_bar_or(false);                   // the previous sweep's keys (or the decisions) are read
+            warps_bar<32 * DW_WARPS>();           // the previous sweep's keys (or the decisions) are read
             // one warp per draw: its descriptor and its z operand
             for (int j = warp; j < DW_NZ; j += DW_WARPS) {
                 DrawDesc dd{};
@@ -814,7 +798,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1) k_acc_draw(AcceptParams p)
                     sh.best[j][0] = sh.best[j][1] = order_key(-INFINITY);
                 }
             }
-            draw_bar_or(false);
+            warps_bar<32 * DW_WARPS>();
             // the target and s words of this lane's draws (16 q + g + 8 h) at ids v, v + 1
             uint32_t tw[2][2], sw[2][2];
             auto fetch = [&](int vb) {
@@ -866,6 +850,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1) k_acc_draw(AcceptParams p)
                 for (int q = 0; q < 2; ++q) {
                     if (16 * q >= nz) break;
                     float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                    __syncwarp();             // the scores of the 16 draws before are taken lane by lane
 #pragma unroll
                     for (int s = 0; s < RANK / 32; ++s) {
                         // physical columns 32 s + 8 t + {0, 1 | 2, 3} are k-step 2 s, + {4, 5 | 6, 7} k-step 2 s + 1
@@ -924,7 +909,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1) k_acc_draw(AcceptParams p)
                         sh.wkey[warp][j][1] = pi[q][h] != 0x7fffffff ? argmax_key(pb[q][h], pi[q][h]) : 0ull;
                     }
                 }
-            if (draw_bar_or(!ok || *abort)) break;
+            if (warps_bar_or<32 * DW_WARPS>(!ok || *abort)) break;
             if ((int)threadIdx.x < 2 * nz) {
                 const int j = threadIdx.x >> 1, hh = threadIdx.x & 1;
                 unsigned long long k = 0ull;

@@ -578,6 +578,34 @@ __device__ __forceinline__ void trace_mark(unsigned long long *tr, int slot, uns
     }
 }
 
+// Warp-collective instructions (.sync.aligned, and the CTA barriers by number)
+// have to be executed by the warp's lanes together.  After a branch that lanes
+// take apart only the compiler's placement would see to that, so each wrapper
+// here rejoins the warp first, and loops of warp-level products do before their
+// first one.
+
+// Barrier 1 over `THREADS` threads (whole warps).
+template <int THREADS> __device__ __forceinline__ void warps_bar()
+{
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+}
+// The same, with the OR of a predicate: all of them take the same decision.
+template <int THREADS> __device__ __forceinline__ bool warps_bar_or(bool pred)
+{
+    uint32_t res;
+    __syncwarp();
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "bar.red.or.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(res)
+        : "r"((uint32_t)pred), "n"(THREADS)
+        : "memory");
+    return res != 0;
+}
+
 // Inter-CTA signalling in global memory at GPU scope.
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p)
 {
@@ -787,16 +815,19 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *map)
 // tcgen05 (5th-generation tensor core, accumulators in tensor memory)
 __device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t ncols)
 {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
                  "r"(ncols)
                  : "memory");
 }
 __device__ __forceinline__ void tmem_relinquish()
 {
+    __syncwarp();
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
 {
+    __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -826,6 +857,7 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
 {
     uint32_t r[32];
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
         "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"

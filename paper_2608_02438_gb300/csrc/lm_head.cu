@@ -72,22 +72,6 @@ static_assert(LmShape<32, 1>::SMEM <= 232448 && LmShape<128, 1>::SMEM <= 232448 
                   LmShape<256, 2>::SMEM <= 232448,
               "shared memory");
 
-// Barrier over the epilogue warps that ORs a predicate (all of them take the
-// same decision to stop).
-template <int WARPS> __device__ __forceinline__ bool lm_epi_bar_or(bool pred)
-{
-    uint32_t res;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, %2, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(res)
-        : "r"((uint32_t)pred), "n"(WARPS * 32)
-        : "memory");
-    return res != 0;
-}
-
 __device__ __forceinline__ bool better(float v, int i, float bv, int bi) { return v > bv || (v == bv && i < bi); }
 
 }  // namespace
@@ -246,7 +230,7 @@ __device__ __forceinline__ void lm_head_body(const CUtensorMap &tmap_w, const CU
                 if (lane == 0) mbar_arrive(&sh.tempty[buf]);
             }
             // the chunk is done in this CTA: its partial per token
-            if (lm_epi_bar_or<Sh::EPI_WARPS>(!got)) break;
+            if (warps_bar_or<32 * Sh::EPI_WARPS>(!got)) break;
             for (int j = threadIdx.x - 64; j < NT; j += Sh::EPI_WARPS * 32) {
                 const int tok = c * NT + j;
                 if (tok < N) {
@@ -258,7 +242,7 @@ __device__ __forceinline__ void lm_head_body(const CUtensorMap &tmap_w, const CU
                     part[(size_t)tok * G + wk.slot] = Partial{a.x, __float_as_int(a.y), 0.0f, 0.0f};
                 }
             }
-            lm_epi_bar_or<Sh::EPI_WARPS>(false);
+            warps_bar<32 * Sh::EPI_WARPS>();
         }
     }
     tc_fence_before();

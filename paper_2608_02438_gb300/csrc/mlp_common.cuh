@@ -54,7 +54,8 @@ __device__ __forceinline__ void bf16x8_to_f32(const uint4 &w, float (&x)[8])
 
 // D (16x8, fp32) += A (16x16, bf16, row-major) * B (16x8, bf16, column-major):
 // the m16n8k16 warp-level tensor-core product (used for the small Trans GEMMs;
-// the vocabulary readout uses tcgen05).
+// the vocabulary readout uses tcgen05).  The caller rejoins the warp before the
+// first of a run of them.
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
     asm volatile(

@@ -78,24 +78,6 @@ static_assert(TC_SMEM_BYTES <= 232448, "k_read_tc shared memory");
 const size_t kReadTcSmemBytes = TC_SMEM_BYTES;
 const int kReadTcThreads = TC_THREADS;
 
-__device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(TC_EPI_WARPS * 32) : "memory"); }
-
-// Named barrier over the 8 epilogue warps that also ORs a predicate, so that
-// every epilogue warp takes the same decision to stop after an abort.
-__device__ __forceinline__ bool epi_bar_or(bool pred)
-{
-    uint32_t res;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, %2, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(res)
-        : "r"((uint32_t)pred), "n"(TC_EPI_WARPS * 32)
-        : "memory");
-    return res != 0;
-}
-
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_read_tc(const Params *__restrict__ pp, const __grid_constant__ CUtensorMap tmap_wr,
               const __grid_constant__ CUtensorMap tmap_z, int V)
@@ -380,9 +362,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 }
             }
             cp_async_wait<0>();                      // nothing in flight into the ring,
-            epi_bar();                               // and every warp is done with its own: the states meet there
+            warps_bar<32 * TC_EPI_WARPS>();                               // and every warp is done with its own: the states meet there
             states[ew][lane] = sel;
-            const bool stop = epi_bar_or(!ok || *abort);
+            const bool stop = warps_bar_or<32 * TC_EPI_WARPS>(!ok || *abort);
             if (!stop) {
                 if (small) {
                     if (ew == 0 && lane < n) {
@@ -396,7 +378,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     p.part[(size_t)i * p.S + r] = a;
                 }
             }
-            epi_bar();
+            warps_bar<32 * TC_EPI_WARPS>();
             if (stop) break;
         }
     }

@@ -601,6 +601,7 @@ __device__ __forceinline__ void mlp_share_mma(const Params &p, cg::cluster_group
     for (int mt = 0; mt * 16 < cnt; ++mt) {
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
         const uint16_t *arow0 = cop + (mt * 16 + g) * COP_LD, *arow1 = arow0 + 8 * COP_LD;
+        __syncwarp();
 #pragma unroll
         for (int ks = 0; ks < RANK / 16; ++ks) {
             uint32_t a[4];
@@ -643,6 +644,7 @@ __device__ __forceinline__ void mlp_share_mma(const Params &p, cg::cluster_group
     for (int mt = 0; mt * 16 < cnt; ++mt) {
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
         const uint16_t *arow0 = uop + (mt * 16 + g) * UOP_LD + khalf * RANK, *arow1 = arow0 + 8 * UOP_LD;
+        __syncwarp();
 #pragma unroll
         for (int ks = 0; ks < RANK / 16; ++ks) {
             uint32_t a[4];

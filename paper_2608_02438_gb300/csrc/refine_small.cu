@@ -294,13 +294,15 @@ __device__ __forceinline__ void pc_consume(const Params &p, uint8_t *ring, RsSha
                     const uint4 al = v ? *reinterpret_cast<const uint4 *>(ft + ml * 128 + ((pc ^ ml) << 4)) : z4;
                     const uint32_t a0[4] = {ah.x, al.x, ah.y, al.y}, a1[4] = {ah.z, al.z, ah.w, al.w};
                     const uint8_t *ht = hb + tile * (NT * 128) + g * 128 + ((pc ^ g) << 4);
+                    uint4 bb[NT / 8];
+#pragma unroll
+                    for (int nt = 0; nt < NT / 8; ++nt)
+                        bb[nt] = (v && nt * 8 + g < N) ? *reinterpret_cast<const uint4 *>(ht + nt * 8 * 128) : z4;
+                    __syncwarp();
 #pragma unroll
                     for (int nt = 0; nt < NT / 8; ++nt) {
-                        const uint4 bb = (v && nt * 8 + g < N)
-                                             ? *reinterpret_cast<const uint4 *>(ht + nt * 8 * 128)
-                                             : z4;
-                        mma_bf16_16816(acc[nt], a0, bb.x, bb.y);
-                        mma_bf16_16816(acc[nt], a1, bb.z, bb.w);
+                        mma_bf16_16816(acc[nt], a0, bb[nt].x, bb[nt].y);
+                        mma_bf16_16816(acc[nt], a1, bb[nt].z, bb[nt].w);
                     }
                 }
             }
@@ -1068,6 +1070,7 @@ __device__ __forceinline__ void trans_role(const Params &p, SmallCtl *c, uint8_t
             for (int mt = 0; mt * 16 < n; ++mt) {
                 float acc[4] = {0.f, 0.f, 0.f, 0.f};
                 const uint16_t *arow0 = cop + (mt * 16 + g) * COP_LD, *arow1 = arow0 + 8 * COP_LD;
+                __syncwarp();
 #pragma unroll
                 for (int ks = 0; ks < RANK / 16; ++ks) {
                     uint32_t a[4];
@@ -1123,6 +1126,7 @@ __device__ __forceinline__ void trans_role(const Params &p, SmallCtl *c, uint8_t
             for (int mt = 0; mt * 16 < n; ++mt) {
                 float acc[4] = {0.f, 0.f, 0.f, 0.f};
                 const uint16_t *arow0 = uop + (mt * 16 + g) * UOP_LD + khalf * RANK, *arow1 = arow0 + 8 * UOP_LD;
+                __syncwarp();
 #pragma unroll
                 for (int ks = 0; ks < RANK / 16; ++ks) {
                     uint32_t a[4];

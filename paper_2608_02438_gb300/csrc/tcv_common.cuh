@@ -47,21 +47,8 @@ __device__ __forceinline__ void tma_load_3d_hint(void *smem_dst, const CUtensorM
         : "memory");
 }
 
-__device__ __forceinline__ void tv_epi_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-
-__device__ __forceinline__ bool tv_epi_bar_or(bool pred)
-{
-    uint32_t res;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, 256, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(res)
-        : "r"((uint32_t)pred)
-        : "memory");
-    return res != 0;
-}
+__device__ __forceinline__ void tv_epi_bar() { warps_bar<256>(); }
+__device__ __forceinline__ bool tv_epi_bar_or(bool pred) { return warps_bar_or<256>(pred); }
 
 // s[v0 .. v0 + 31] of one token as raw bf16 pairs (zeros past V or for an
 // invalid lane).

@@ -104,11 +104,6 @@ static_assert(tr_stages(TR_STATS) <= TR_SMAX && tr_stages(TR_TV) >= 2 && tr_stag
                   tr_stages(TR_TV) <= TR_SMAX && tr_stages(TR_DZ) <= TR_SMAX && tr_bstages(TR_DZ) <= TR_BMAX,
               "ring depths");
 
-__device__ __forceinline__ void tr_epi_bar()
-{
-    asm volatile("bar.sync 1, %0;" ::"n"(TR_EPI_WARPS * 32) : "memory");
-}
-
 // log2-domain running log-sum-exp over 16 values (as pairs): value = s * 2^m.
 // The max and the sum run as trees (short dependent chains).
 __device__ __forceinline__ void lse2_add16(float &m, float &s, const unsigned long long (&x)[8])
@@ -586,11 +581,11 @@ __device__ __forceinline__ void train_tok_body(const TrainParams &p, const CUten
             f32x2_split(r3, lo[2], hi[2]);
             const float4 o4 = mode == TR_STATS ? make_float4(m2, s2, 0.f, 0.f)
                                                : make_float4(lo[0] + hi[0], lo[1] + hi[1], 0.f, lo[2] + hi[2]);
-            tr_epi_bar();
+            warps_bar<32 * TR_EPI_WARPS>();
             float4 *scr = reinterpret_cast<float4 *>(sS);
             const int slot = 2 * set + g;
             if (slot != 0) scr[(slot - 1) * TR_BM + row] = o4;
-            tr_epi_bar();
+            warps_bar<32 * TR_EPI_WARPS>();
             if (slot == 0 && valid && ok && !*abort) {
                 float4 a = o4;
                 for (int k = 0; k < 3; ++k) {

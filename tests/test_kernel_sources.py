@@ -4,6 +4,8 @@ A bounded wait may run out in one lane (or see the abort there) while its
 neighbours' succeed.  Where a warp goes on to warp-collective instructions, its
 lanes must not part over that: such a wait is taken by ``mbar_wait_warp`` /
 ``mbar_wait_spin_warp``, and the per-thread forms are left to single threads.
+Lanes that took a branch apart meet again before the next such instruction:
+inside its wrapper, or before a run of warp-level products.
 """
 import os
 import re
@@ -78,3 +80,33 @@ def test_waits_of_a_whole_warp_are_taken_together():
             line = text.count("\n", 0, m.start()) + 1
             assert _single_thread(sources, name, m.start()), f"{name}:{line}: a per-thread wait outside a single thread"
     assert found > 30
+
+
+def test_warp_collective_instructions_rejoin_the_warp_first():
+    found = 0
+    for f in sorted(os.listdir(CSRC)):
+        if not f.endswith((".cu", ".cuh")):
+            continue
+        with open(os.path.join(CSRC, f)) as fh:
+            text = fh.read()
+        for m in re.finditer(r"tcgen05\.(?:ld|st|alloc|dealloc|relinquish_alloc_permit)\.[\w.:]*sync\.aligned|\bbar\.(?:sync|red)\b",
+                             text):
+            found += 1
+            body = text[text.rindex("__device__ __forceinline__", 0, m.start()):m.start()]
+            line = text.count("\n", 0, m.start()) + 1
+            assert "__syncwarp();" in body, f"{f}:{line}: {m.group(0)} does not rejoin the warp"
+    assert found >= 8
+
+
+def test_warp_level_products_start_from_a_joined_warp():
+    found = 0
+    for name, text in _sources().items():
+        for m in re.finditer(r"\bmma_bf16_16816\(", text):
+            before = text[:m.start()]
+            if before.endswith("void "):
+                continue                                 # the definition
+            found += 1
+            line = before.count("\n") + 1
+            at = before.rfind("__syncwarp();")
+            assert at >= 0 and not re.search(r"\bif \(|\?", before[at:]), f"{name}:{line}: a branch since the warp met"
+    assert found >= 8
