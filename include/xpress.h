@@ -334,7 +334,8 @@ size_t xpress_train_workspace_size(const xpress_refiner *refiner, int b, int B);
  * total-variation sums, dL/dz with dL/dl stored --, the product dL/dW_r of the
  * stored dL/dl with z, and the backward products; that product and some of the
  * weight gradients run on streams of the refiner's own, forked from `stream`
- * and joined before the call returns, also under stream capture).  Token
+ * and joined before the call returns, with an error too, also under stream
+ * capture).  Token
  * ids out of [0, V) are clamped to 0 and reported by the status word
  * (XPRESS_ERR_DEVICE_CHECK); a bounded wait that gives up reports
  * XPRESS_ERR_TIMEOUT there.

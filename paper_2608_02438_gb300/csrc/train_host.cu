@@ -10,6 +10,7 @@
 #include <cstdint>
 #include <mutex>
 
+#include "fork_join.h"
 #include "kernels.h"
 #include "xpress.h"
 
@@ -407,9 +408,12 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
     XT_CUDA(launch(k_train_tok_tv, gtok, dim3(kTrainTokThreads), kTrainTokSmemBytes, st, tp, tz128, tw64, ts64,
                    tt64));
     XT_CUDA(launch(k_train_tv_fin, dim3(in->b), dim3(32, in->B), 0, st, m));
+    // The refiner's own streams beside `st`: one for the dL/dW_r product, one for
+    // the other weight gradients.  Both are joined however the call ends.
     cudaEvent_t ev[5];
-    cudaStream_t dws;
-    const cudaStream_t aux = refiner_train_aux(R, dws, ev);
+    cudaStream_t dw_stream;
+    const cudaStream_t aux = refiner_train_aux(R, dw_stream, ev);
+    StreamFork dw_fork(st, dw_stream, ev[4]), aux_fork(st, aux, ev[3]);
     for (int j0 = 0; j0 < mt; j0 += L.dl_tiles) {
         const int n = mt - j0 < L.dl_tiles ? mt - j0 : L.dl_tiles;
         XT_CUDA(run_dz(j0, n));
@@ -422,9 +426,8 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
         // latency-bound kernels: TRAIN_DW_LEAVE SMs stay free for their products
         // (the others' shared memory is taken), and the HBM-bound product does
         // not need them.  Both add into gW_r atomically.
-        XT_CUDA(cudaEventRecord(ev[4], st));
-        XT_CUDA(cudaStreamWaitEvent(dws, ev[4], 0));
-        XT_CUDA(run_dw(j0, n, dws, sms > 2 * TRAIN_DW_LEAVE ? sms - TRAIN_DW_LEAVE : sms));
+        XT_CUDA(dw_fork.fork(ev[4]));
+        XT_CUDA(run_dw(j0, n, dw_stream, sms > 2 * TRAIN_DW_LEAVE ? sms - TRAIN_DW_LEAVE : sms));
     }
 
     // backward through Trans (Eq. mlp)
@@ -433,12 +436,10 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
                    F(L.du), 2 * r, nullptr, 0, nullptr, 0, 0)))
         return rc;
     XT_CUDA(launch(k_train_dact, dim3((NR * 2 * r / 4 + 255) / 256), dim3(256), 0, st, m));
-    // The weight-gradient products run on the refiner's second stream beside
-    // the input-gradient chain (dz -> dc -> Mix backward -> dX -> Fuse
-    // backward), each forked once its operands exist and joined at the end;
-    // none of their operands is written again in the step.
-    XT_CUDA(cudaEventRecord(ev[0], st));                        // dz and dt
-    XT_CUDA(cudaStreamWaitEvent(aux, ev[0], 0));
+    // The weight-gradient products run beside the input-gradient chain (dz -> dc
+    // -> Mix backward -> dX -> Fuse backward), each forked once its operands
+    // exist; none of their operands is written again in the step.
+    XT_CUDA(aux_fork.fork(ev[0]));                              // dz and dt
     if ((rc = gemm(aux, sms, r, 2 * r, NR, {U(L.dzb), (uint64_t)r, true}, {U(L.uop), (uint64_t)2 * r, true}, GM_ADD,
                    1.f, out->gW2, 2 * r, nullptr, 0, nullptr, 0, 0)))
         return rc;
@@ -451,8 +452,7 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
 
     // backward through Mix (Eq. mix) and Fuse (Eq. fuse)
     XT_CUDA(launch(k_train_mix_bwd, gmix, bmix, train_mix_smem(in->B), st, m));
-    XT_CUDA(cudaEventRecord(ev[1], st));                        // dL/da
-    XT_CUDA(cudaStreamWaitEvent(aux, ev[1], 0));
+    XT_CUDA(aux_fork.fork(ev[1]));                              // dL/da
     if ((rc = gemm(aux, sms, r, 3 * r, NR, {U(L.dab), (uint64_t)r, true}, {U(L.X), (uint64_t)5 * r, true}, GM_ADD, 1.f,
                    out->gW_in, 3 * r, nullptr, 0, nullptr, 0, 0)))
         return rc;
@@ -460,18 +460,15 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
                    1.f, F(L.dX), 3 * r, nullptr, 0, nullptr, 0, 0)))
         return rc;
     XT_CUDA(launch(k_train_fuse_bwd, dim3(P), dim3(RANK), 0, st, m));
-    XT_CUDA(cudaEventRecord(ev[2], st));                        // dL/du_h, dL/du_g
-    XT_CUDA(cudaStreamWaitEvent(aux, ev[2], 0));
+    XT_CUDA(aux_fork.fork(ev[2]));                              // dL/du_h, dL/du_g
     if ((rc = gemm(aux, sms, r, H, P, {U(L.D) + r, (uint64_t)2 * r, true}, h_mn, GM_ADD, 1.f, out->gW_g, H, nullptr, 0,
                    nullptr, 0, 0)))
         return rc;
     if ((rc = gemm(st, sms, r, H, P, {U(L.D), (uint64_t)2 * r, true}, h_mn, GM_ADD, 1.f, out->gW_h, H, nullptr, 0,
                    nullptr, 0, 0)))
         return rc;
-    XT_CUDA(cudaEventRecord(ev[3], aux));                       // join both
-    XT_CUDA(cudaStreamWaitEvent(st, ev[3], 0));
-    XT_CUDA(cudaEventRecord(ev[4], dws));
-    XT_CUDA(cudaStreamWaitEvent(st, ev[4], 0));
+    XT_CUDA(aux_fork.join());
+    XT_CUDA(dw_fork.join());
     return XPRESS_OK;
 }
 
