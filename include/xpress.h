@@ -315,7 +315,8 @@ typedef struct {
 
 /* Gradients are ADDED into the caller's fp32 buffers (zero them to start a
  * step; leave them to accumulate over several batches), each shaped like its
- * weight (xpress_weights); gL's upper triangle and diagonal are left alone.
+ * weight (xpress_weights); gW_r 16-byte aligned, the others at any 4-byte
+ * boundary; gL's upper triangle and diagonal are left alone.
  * loss: [b, 4] per block L(p^r), L(p^b), L(p^r-hat), L_total (overwritten). */
 typedef struct {
     float *loss;
@@ -335,11 +336,10 @@ size_t xpress_train_workspace_size(const xpress_refiner *refiner, int b, int B);
  * stored dL/dl with z, and the backward products; that product and some of the
  * weight gradients run on streams of the refiner's own, forked from `stream`
  * and joined before the call returns, with an error too, also under stream
- * capture).  Token
- * ids out of [0, V) are clamped to 0 and reported by the status word
- * (XPRESS_ERR_DEVICE_CHECK); a bounded wait that gives up reports
+ * capture).  Token ids out of [0, V) are clamped to 0 and reported by the status
+ * word (XPRESS_ERR_DEVICE_CHECK); a bounded wait that gives up reports
  * XPRESS_ERR_TIMEOUT there.
- * Errors: INVALID_ARG (NULL pointer, h / s / target not 16-byte aligned,
+ * Errors: INVALID_ARG (NULL pointer, h / s / target / gW_r not 16-byte aligned,
  * b < 1, B mismatch, gamma <= 0), UNSUPPORTED (fp32 refiner), WORKSPACE, CUDA. */
 int xpress_train_step(const xpress_refiner *refiner, const xpress_train_in *in, const xpress_train_out *out,
                       void *workspace, size_t ws_bytes, void *stream);

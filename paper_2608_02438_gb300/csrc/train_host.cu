@@ -227,9 +227,10 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
         !(in->gamma > 0.0f) || !out->loss || !out->gW_e || !out->gW_h || !out->gW_g || !out->gW_in || !out->gL ||
         !out->gW1 || !out->gW2 || !out->gW_r)
         return XPRESS_ERR_INVALID_ARG;
-    // h, s and target are read by bulk copies, tensor maps and 16-byte loads
+    // h, s and target are read by bulk copies, tensor maps and 16-byte loads, gW_r
+    // is added into by bulk tensor reductions
     if (((reinterpret_cast<uintptr_t>(in->h) | reinterpret_cast<uintptr_t>(in->s) |
-          reinterpret_cast<uintptr_t>(in->target)) & 15) != 0)
+          reinterpret_cast<uintptr_t>(in->target) | reinterpret_cast<uintptr_t>(out->gW_r)) & 15) != 0)
         return XPRESS_ERR_INVALID_ARG;
     if (refiner_device(R) >= 0) {
         int dev = -1;

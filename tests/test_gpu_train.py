@@ -178,3 +178,28 @@ def test_train_step_rejects(X):
         ref.train_step(torch.zeros((1, 8, 128), device="cuda"), f, f, z, z[:1])
     assert err.value.code == X.XPRESS_ERR_UNSUPPORTED
     ref.close()
+
+
+# dL/dW_r is added by bulk tensor reductions: its buffer must sit at a 16-byte
+# boundary.  The other gradients may be views at any 4-byte one.
+def test_train_step_gradient_alignment(X):
+    cfg = W.tiny_config("tral", b=3, B=8, H=136, V=1032, r=256, dtype=W.BF16, seed=4500)
+    w = W.make_weights(cfg.H, cfg.V, cfg.r, cfg.B, cfg.dtype, 4501, "paper")
+    inp = W.make_train_inputs(cfg)
+    ref = X.Refiner({k: _bf16_dev(X, v) for k, v in w.items()}, cfg.H, cfg.V, cfg.r, cfg.B, X.XPRESS_BF16)
+    args = [_bf16_dev(X, inp[k]) for k in ("h", "s", "target")] + [torch.from_numpy(inp[k]).cuda()
+                                                                  for k in ("ystar", "anchor")]
+
+    def shifted(t):
+        return torch.zeros(t.numel() + 4, dtype=t.dtype, device="cuda")[1:1 + t.numel()].view(t.shape)
+
+    _, grads = ref.train_step(*args)
+    moved = {k: shifted(v) if k != "W_r" else torch.zeros_like(v) for k, v in grads.items()}
+    ref.train_step(*args, grads=moved)
+    torch.cuda.synchronize()
+    for k, v in grads.items():
+        np.testing.assert_allclose(moved[k].cpu().numpy(), v.cpu().numpy(), rtol=1e-5, atol=1e-6 * float(v.abs().max()))
+    with pytest.raises(X.XpressError) as err:
+        ref.train_step(*args, grads={**grads, "W_r": shifted(grads["W_r"])})
+    assert err.value.code == X.XPRESS_ERR_INVALID_ARG
+    ref.close()
