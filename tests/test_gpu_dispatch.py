@@ -227,3 +227,33 @@ def test_read_token_tiles(X, b, B, V):
         orc = dict(enumerate(ex.map(lambda i: run_oracle(m, inp, i, cfg.K_max, False), range(b))))
     g = {k: (v.cpu().numpy() if v is not None else None) for k, v in out.items()}
     compare_blocks(g, orc, list(range(b)), cfg.dtype, m=m, inp=inp)
+
+
+# The hidden projection of the graph path (k_pre_tc), alone: W_in picks
+# F = W_h + 2^-8 (W_h one row on), exact in the hi and lo terms, and everything
+# after it is zero, so z = F h.  An accumulation step in tensor memory cuts the sum
+# off by up to 2^-23 of it, 2^-24 on average; an accumulator takes n steps of 16
+# products of the hi term (8 where 16 slices of 256 go to two accumulators, 28 for
+# slices of 13 chunks of 64), and its sum grows to the end: below n 2^-24.
+@pytest.mark.parametrize("b,B,n", [(3, 16, 8), (20, 16, 8), (64, 32, 28)])
+def test_hidden_projection_accuracy(X, b, B, n):
+    H, V, r = 4096, 64, 256
+    g = torch.Generator(device="cuda").manual_seed(b)
+
+    def zeros(*shape):
+        return torch.zeros(shape, dtype=torch.bfloat16, device="cuda")
+
+    W_h = (torch.randint(8, 16, (r, H), generator=g, device="cuda").float() / 8).bfloat16()
+    W_in = zeros(r, 3 * r)
+    W_in[:, :r] = (torch.eye(r) + torch.roll(torch.eye(r), 1, 1) * 2.0 ** -8).cuda()
+    ref = X.Refiner(dict(W_e=zeros(V, r), W_h=W_h, W_g=zeros(r, H), W_in=W_in, L=zeros(r, B, B), W1=zeros(2 * r, r),
+                         W2=zeros(r, 2 * r), W_r=zeros(V, r)), H, V, r, B, X.XPRESS_BF16)
+    h = torch.randn((b, B, H), generator=g, device="cuda").bfloat16()
+    s = torch.randn((b, B, V), generator=g, device="cuda").bfloat16()
+    i32 = dict(dtype=torch.int32, device="cuda")
+    out = ref.refine_block(h, s, torch.zeros((b, B), **i32), torch.zeros(b, **i32), torch.zeros(b, device="cuda"),
+                           torch.zeros(b, dtype=torch.int64, device="cuda"), 1, 2)
+    torch.cuda.synchronize()
+    assert ref.device_status("refine", b) == X.XPRESS_OK
+    exact = h.double() @ (W_in.double()[:, :r] @ W_h.double()).T
+    assert float((out["z_final"].double() - exact).norm() / exact.norm()) < n * 2.0 ** -24
