@@ -5,20 +5,21 @@
 // GEMM view: D[v, t] = W_lm[v, :] . h[t, :], M = MT tiles of 128 vocabulary
 // rows (the weight stream, 1.245 GB at the Qwen3-8B shape), N = NT tokens (a
 // chunk of the N hidden states), K = H.  Vocabulary rows sit in TMEM lanes, so
-// the stores of s are runs of 64 bytes per token.  With NC chunks, CTA r works on
-// chunk r % NC and takes every Gc-th vocabulary item of it (Gc CTAs per chunk), so
-// that the NC CTAs of an item read the same rows of W_lm at about the same time:
-// one read from HBM, the others from L2.
+// the stores of s are runs of 64 bytes per token.  Up to 16 chunks at a time share
+// the CTAs (LmWork), so that the CTAs of an item read the same rows of W_lm at about
+// the same time: one read from HBM, the others from L2.
 //
 // Tiles by N (lm_shape): up to 32 tokens NT = 32, up to 128 NT = 128 (both
 // HBM-bound on W_lm: the smaller the token part of a ring stage, the more of W_lm
 // is in flight; 83 tokens 204 us against 236 in a 256-token chunk);
 // beyond, NT = 256, where both operands come from L2 and tensor time and the
 // L2-to-SM stream compete: MT = 2 loads 64 KB per 256 x 256 x 64 product instead
-// of 48 KB per 128 x 256 x 64 (512 tokens 445 us against 454 with MT = 1 and 548
-// with whole chunks one after the other, W_lm from HBM for each; 433 without the
-// stores of s), at the price of a single accumulator (the epilogue is not
-// overlapped).  MT = 1 remains where MT = 2 leaves CTAs without an item.
+// of 48 KB per 128 x 256 x 64, at the price of a single accumulator (the epilogue is
+// not overlapped).  Measured at the Qwen3-8B shape, MT = 2 / MT = 1 / MT = 1 and
+// whole chunks one after the other, us: 129 tokens 215 / 216 / 216, 160 220 / 225 /
+// 225, 256 255 / 255 / 256, 300 410 / 395 / 466, 384 393 / 415 / 483, 512 445 / 454 /
+// 540, 1024 880 / 905 / 1065, 2048 1655 / 1740 / 2110 (512 without the stores of s:
+// 433).  MT = 1 remains where MT = 2 would leave fewer than two items per CTA.
 //
 // Roles (32 (2 + 4 MT) threads):
 //   warp 0     TMA producer: per K-chunk of 64, a 128 MT x 64 box of W_lm and an
@@ -35,6 +36,7 @@
 // kernel combines the partials of each token (ties: smallest id).
 #include "train_common.cuh"
 #include "kernels.h"
+#include "lm_work.h"
 
 namespace xp {
 
@@ -76,21 +78,6 @@ __device__ __forceinline__ bool better(float v, int i, float bv, int bi) { retur
 
 }  // namespace
 
-// The items of CTA r of G: chunk chunk0 (and, when there are more chunks than
-// CTAs, every G-th one after it), vocabulary items first, first + step, ...; its
-// partials go to slot `slot` of a token's G.
-struct LmWork {
-    int chunk0, chunk_step, first, step, slot;
-    __device__ __forceinline__ LmWork(int r, int G, int NC)
-    {
-        if (NC <= G) {
-            chunk0 = r % NC; chunk_step = NC; first = slot = r / NC; step = (G - 1 - chunk0) / NC + 1;
-        } else {
-            chunk0 = r; chunk_step = G; first = slot = 0; step = 1;
-        }
-    }
-};
-
 // grid G <= NC x items (every CTA has an item), LmShape::THREADS threads, LmShape::SMEM bytes.
 template <int NT, int MT>
 __device__ __forceinline__ void lm_head_body(const CUtensorMap &tmap_w, const CUtensorMap &tmap_h, int V, int H, int N,
@@ -130,8 +117,9 @@ __device__ __forceinline__ void lm_head_body(const CUtensorMap &tmap_w, const CU
             int stage = 0;
             uint32_t phase = 0, pending = 0, pend_par = 0;
             bool ok = true;
-            for (int c = wk.chunk0; c < NC && ok; c += wk.chunk_step)
-                for (int it = wk.first; it < NI && ok; it += wk.step)
+            for (int gr = 0; gr < wk.groups && ok; ++gr) {
+                const int c = wk.chunk(gr), step = wk.step(gr);
+                for (int it = wk.first(gr); it < NI && ok; it += step)
                     for (int kc = 0; kc < KCH; ++kc) {
                         if (!mbar_wait(&sh.empty[stage], phase ^ 1, abort)) { ok = false; break; }
                         uint8_t *dst = base + stage * Sh::STAGE;
@@ -142,6 +130,7 @@ __device__ __forceinline__ void lm_head_body(const CUtensorMap &tmap_w, const CU
                         pend_par = (pend_par & ~(1u << stage)) | (phase << stage);
                         if (++stage == Sh::STAGES) { stage = 0; phase ^= 1; }
                     }
+            }
             // no copy may still be landing when the CTA leaves
             int dummy = 0;
             for (int st = 0; st < Sh::STAGES; ++st)
@@ -155,8 +144,9 @@ __device__ __forceinline__ void lm_head_body(const CUtensorMap &tmap_w, const CU
             int stage = 0, t = 0;
             uint32_t phase = 0;
             bool ok = true;
-            for (int c = wk.chunk0; c < NC && ok; c += wk.chunk_step)
-                for (int it = wk.first; it < NI && ok; it += wk.step, ++t) {
+            for (int gr = 0; gr < wk.groups && ok; ++gr) {
+                const int step = wk.step(gr);
+                for (int it = wk.first(gr); it < NI && ok; it += step, ++t) {
                     const int buf = t % Sh::NBUF;
                     if (!mbar_wait(&sh.tempty[buf], ((t / Sh::NBUF) & 1) ^ 1, abort)) { ok = false; break; }
                     tc_fence_after();
@@ -176,6 +166,7 @@ __device__ __forceinline__ void lm_head_body(const CUtensorMap &tmap_w, const CU
                     }
                     if (ok) tc_commit(&sh.tfull[buf]);
                 }
+            }
             tc_commit(&sh.drain);
             int dummy = 0;
             mbar_wait(&sh.drain, 0, &dummy, 100000000ull);
@@ -188,11 +179,12 @@ __device__ __forceinline__ void lm_head_body(const CUtensorMap &tmap_w, const CU
         float2 *best = reinterpret_cast<float2 *>(scratch + Sh::TILE_BYTES);   // [warp][NT] (value, id bits)
         int t = 0;
         bool got = true;
-        for (int c = wk.chunk0; c < NC && got; c += wk.chunk_step) {
+        for (int gr = 0; gr < wk.groups && got; ++gr) {
+            const int c = wk.chunk(gr), slot = wk.first(gr), step = wk.step(gr);
 #pragma unroll 1
             for (int g = 0; g < NT / 32; ++g)
                 best[ew * NT + g * 32 + lane] = make_float2(-INFINITY, __int_as_float(0x7fffffff));
-            for (int it = wk.first; it < NI && got; it += wk.step, ++t) {
+            for (int it = slot; it < NI && got; it += step, ++t) {
                 const int buf = t % Sh::NBUF;
                 got = mbar_wait_warp(&sh.tfull[buf], (t / Sh::NBUF) & 1, abort);
                 tc_fence_after();
@@ -239,7 +231,7 @@ __device__ __forceinline__ void lm_head_body(const CUtensorMap &tmap_w, const CU
                         const float2 b = best[w * NT + j];
                         if (better(b.x, __float_as_int(b.y), a.x, __float_as_int(a.y))) a = b;
                     }
-                    part[(size_t)tok * G + wk.slot] = Partial{a.x, __float_as_int(a.y), 0.0f, 0.0f};
+                    part[(size_t)tok * G + slot] = Partial{a.x, __float_as_int(a.y), 0.0f, 0.0f};
                 }
             }
             warps_bar<32 * Sh::EPI_WARPS>();
@@ -263,7 +255,7 @@ __global__ void __launch_bounds__(256) k_lm_head_argmax(const Partial *part, int
     const int tok = blockIdx.x * 8 + threadIdx.x / 32, lane = threadIdx.x % 32;
     if (tok >= N) return;
     const int NC = (N + NT - 1) / NT, c = tok / NT;
-    const int slots = LmWork(NC <= G ? c : c % G, G, NC).step;         // CTAs that worked on the token's chunk
+    const int slots = LmWork(0, G, NC).slots(c);                       // CTAs that worked on the token's chunk
     float m = -INFINITY;
     int mi = 0x7fffffff;
     for (int s = lane; s < slots; s += 32) {

@@ -257,3 +257,10 @@ def test_hidden_projection_accuracy(X, b, B, n):
     assert ref.device_status("refine", b) == X.XPRESS_OK
     exact = h.double() @ (W_in.double()[:, :r] @ W_h.double()).T
     assert float((out["z_final"].double() - exact).norm() / exact.norm()) < n * 2.0 ** -24
+
+
+# More token chunks than a group of the LM head holds, and more than CTAs: 17
+# (eight and nine) over 41 CTAs, 19 over four (five groups) and 300 over two.
+@pytest.mark.parametrize("N,V,H", [(4100, 5128, 72), (4650, 392, 64), (76570, 136, 64)])
+def test_lm_head_chunk_groups(X, N, V, H):
+    test_lm_head_shapes(X, N, V, H)
