@@ -387,7 +387,7 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
     if ((rc = gemm(st, sms, P, r, H, h_k, {w.W_g, (uint64_t)H, false}, GM_PART, 1.f, F(L.Ug), r, nullptr, 0, nullptr,
                    0, 0)))
         return rc;
-    XT_CUDA(launch(k_train_fuse, dim3(r / 32, in->b + (NR / 2 - P + in->B - 1) / in->B), dim3(32, in->B), 0, st, m));
+    XT_CUDA(launch(k_train_fuse, dim3(in->b + (NR / 2 - P + in->B - 1) / in->B, r / 32), dim3(32, in->B), 0, st, m));
     // one product over [X | lo parts of u_h and u_g], the latter against W_in[:, 0:2r] again
     if ((rc = gemm(st, sms, NR, r, 5 * r, {U(L.X), (uint64_t)5 * r, false}, {w.W_in, (uint64_t)3 * r, false}, GM_STORE,
                    1.f, F(L.a), r, nullptr, 0, nullptr, 0, 0, 3 * r)))

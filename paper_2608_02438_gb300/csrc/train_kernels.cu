@@ -309,8 +309,8 @@ __global__ void __launch_bounds__(256) k_train_rows_fin(TrainMisc m)
     }
 }
 
-// grid (r / 32, b + ceil((NR / 2 - P) / B)), block (32, B): channel d0 + x,
-// position y of block blockIdx.y (past b: a padding position, zeroed).
+// grid (b + ceil((NR / 2 - P) / B), r / 32), block (32, B): position y of block
+// blockIdx.x (past b: a padding position, zeroed), channel 32 blockIdx.y + x.
 // Latency-bound on the K-split slices of W_h h and W_g h, at most 152 of each
 // per element: every (position, channel) has its own thread, which requests its
 // slices together and adds them in a fixed order (with 256 threads per four
@@ -321,8 +321,8 @@ __global__ void __launch_bounds__(1024) k_train_fuse(TrainMisc m)
 {
     pdl_trigger();
     pdl_wait();
-    const int d = blockIdx.x * 32 + threadIdx.x, k = threadIdx.y, B = m.B, r5 = 5 * RANK;
-    const int blk = blockIdx.y;
+    const int d = blockIdx.y * 32 + threadIdx.x, k = threadIdx.y, B = m.B, r5 = 5 * RANK;
+    const int blk = blockIdx.x;
     if (blk >= m.b) {
         // padding rows: zero operands and activations so that every product
         // over them vanishes

@@ -264,3 +264,22 @@ def test_hidden_projection_accuracy(X, b, B, n):
 @pytest.mark.parametrize("N,V,H", [(4100, 5128, 72), (4650, 392, 64), (76570, 136, 64)])
 def test_lm_head_chunk_groups(X, N, V, H):
     test_lm_head_shapes(X, N, V, H)
+
+
+# More blocks than a grid holds in y, and a ragged last row tile: the step is
+# accepted and is the sum of the steps of its two halves (to the bound of
+# test_train_row_tile_groups).
+def test_train_many_short_blocks(X):
+    cfg = W.Config("train_many", b=65520, B=2, H=64, V=64, r=256, dtype=W.BF16, K_max=2, logits="gauss4_spike", seed=93)
+    ref, dt = _refiner(X, cfg, W.make_weights(cfg.H, cfg.V, cfg.r, cfg.B, cfg.dtype, 94, "paper"))
+    inp = W.make_train_inputs(cfg)
+    args = [X.to_device(inp[k], dt) for k in ("h", "s", "target")] + [torch.from_numpy(inp[k]).cuda()
+                                                                     for k in ("ystar", "anchor")]
+    loss, grads = ref.train_step(*args)
+    n, halves = cfg.b // 2, ref.alloc_grads()
+    parts = [ref.train_step(*(a[j].contiguous() for a in args), grads=halves)[0] for j in (slice(0, n), slice(n, cfg.b))]
+    torch.cuda.synchronize()
+    assert ref.device_status("train", cfg.b) == X.XPRESS_OK
+    assert torch.allclose(loss, torch.cat(parts), rtol=1e-5, atol=1e-4)
+    for k, g in grads.items():
+        assert float((g - halves[k]).norm() / halves[k].norm()) < 6 * 2.0 ** -13, k
