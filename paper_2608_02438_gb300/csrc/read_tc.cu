@@ -150,11 +150,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     if (warp == 0) {
         // ------------------------------------------------------- producer
         if (lane == 0) {
-            int stage = 0, skip = pre;
+            int stage = 0, skip = pre, a_tiles = 0;
             uint32_t phase = 0, pending = 0, pend_par = 0;
             for (int i = 0; i < pre; ++i) pending |= 1u << i;
             for (int j = 0; j < MT && !*abort; ++j) {
                 if (!mbar_wait(&sh.a_empty, (j & 1) ^ 1, abort)) break;
+                a_tiles = j + 1;
                 mbar_expect_tx(&sh.a_full, TC_A_BYTES);
                 for (int kc = 0; kc < TC_KCH; ++kc)
                     for (int q = 0; q < 4; ++q)
@@ -178,11 +179,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             }
             if (*abort) {
                 // let the copies already issued land before the CTA goes away
+                int dummy = 0;
                 for (int st = 0; st < TC_STAGES; ++st)
-                    if (pending & (1u << st)) {
-                        int dummy = 0;
-                        mbar_wait(&sh.full[st], (pend_par >> st) & 1, &dummy, 10000000ull);
-                    }
+                    if (pending & (1u << st)) mbar_wait(&sh.full[st], (pend_par >> st) & 1, &dummy, 10000000ull);
+                if (a_tiles) mbar_wait(&sh.a_full, (a_tiles - 1) & 1, &dummy, 10000000ull);
             }
         }
     } else if (warp == 1) {

@@ -5,7 +5,8 @@ neighbours' succeed.  Where a warp goes on to warp-collective instructions, its
 lanes must not part over that: such a wait is taken by ``mbar_wait_warp`` /
 ``mbar_wait_spin_warp``, and the per-thread forms are left to single threads.
 Lanes that took a branch apart meet again before the next such instruction:
-inside its wrapper, or before a run of warp-level products.
+inside its wrapper, or before a run of warp-level products.  And no bulk copy may
+still be landing in a CTA's shared memory when the CTA leaves.
 """
 import os
 import re
@@ -110,3 +111,13 @@ def test_warp_level_products_start_from_a_joined_warp():
             at = before.rfind("__syncwarp();")
             assert at >= 0 and not re.search(r"\bif \(|\?", before[at:]), f"{name}:{line}: a branch since the warp met"
     assert found >= 8
+
+
+def test_every_copy_is_drained_when_a_kernel_gives_up():
+    kernels = 0
+    for name, text in _sources().items():
+        copies = set(re.findall(r"mbar_expect_tx\(&sh\.(\w+)", text))
+        drained = set(re.findall(r"mbar_wait(?:_spin)?\(&sh\.(\w+)[^;]*&dummy", text))
+        kernels += bool(copies)
+        assert copies <= drained, f"{name}: {sorted(copies - drained)} may still be landing"
+    assert kernels >= 9
