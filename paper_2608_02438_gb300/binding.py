@@ -283,11 +283,22 @@ class Refiner:
         except Exception:
             pass
 
+    @staticmethod
+    def train_workspace_sizes(b: int) -> range:
+        """The batch sizes that share a training workspace with b: eight groups per
+        octave.  The workspace takes near a gigabyte per thousand positions of a
+        large vocabulary, and none is given back while the refiner lives (a
+        captured step holds its address), so a loop over many batch sizes is left
+        with about 12 times the largest."""
+        step = 1 << max(0, (b - 1).bit_length() - 4)
+        last = -(-b // step) * step
+        return range(last - step + 1, last + 1)
+
     def workspace(self, kind: str, b: int):
-        key = (kind, b)
+        key = (kind, b if kind != "train" else self.train_workspace_sizes(b)[-1])
         if key not in self._ws:
             if kind == "train":
-                size = xpress_train_workspace_size(self.handle, b, self.B)
+                size = max(xpress_train_workspace_size(self.handle, q, self.B) for q in self.train_workspace_sizes(b))
             else:
                 size = (xpress_refine_workspace_size if kind == "refine" else xpress_accept_workspace_size)(
                     self.handle, b)
@@ -372,6 +383,8 @@ class Refiner:
         return loss, grads
 
     def device_status(self, kind: str = "refine", b: int = 1) -> int:
+        """The device status of the last call on the workspace of that kind and
+        batch size (training: shared by the sizes of train_workspace_sizes)."""
         ws, _ = self.workspace(kind, b)
         return xpress_get_device_status(ws, self.stream.cuda_stream)
 
