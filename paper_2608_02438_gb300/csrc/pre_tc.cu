@@ -6,11 +6,13 @@
 // Fuse/Mix precompute).  F is stored as two bf16 terms hi + lo, run as a
 // doubled K loop: bf16 operands (exact products), fp32 accumulation in TMEM.
 // Every step of that accumulation cuts the sum off, so the error grows with the
-// steps taken on a full-sized sum.  The lo terms come first (their sums are 2^-8 of
-// the result) and the K-chunks go to two accumulators in turn, which the epilogue
-// adds: a relative error of 1.1e-7 at 80 tokens and 2.5e-7 at 2048 (H = 4096,
-// normal inputs), against 6.3e-7 and 2.1e-6 with one accumulator and hi first, and
-// 2.1e-7 with K cut into 64 slices at 80 tokens.
+// steps taken on a full-sized sum.  Up to PT_PAIRED_TILES token tiles, where the cap on
+// the K slices makes them longer than one wave of CTAs would, the lo terms come
+// first (their sums are 2^-8 of the result) and the K-chunks go to two accumulators
+// in turn, which the epilogue adds: a relative error of 1.1e-7 at 80 tokens (H = 4096,
+// normal inputs) against 6.3e-7 with hi first and one accumulator, and 2.1e-7 without
+// the cap (64 slices).  Larger batches, whose slices the cap does not touch, run hi
+// first into one (2.1e-6 at 2048 tokens, 5 slices), bit for bit as without it.
 // Each CTA computes one 128-token x 256-row tile over one K-slice and writes it
 // as a split-K partial Upart[slice][t][o].
 //
@@ -28,7 +30,7 @@ constexpr int PT_BM = 128;                    // tokens (M)
 constexpr int PT_BN = 256;                    // rows of W_h or W_g (N)
 constexpr int PT_BK = 64;
 constexpr int PT_STAGES = 4;
-constexpr int PT_NACC = 2;                    // accumulators, K-chunks dealt to them in turn
+constexpr int PT_PAIRED_TILES = 4;            // most token tiles with two accumulators
 constexpr uint32_t PT_A_STAGE = PT_BM * PT_BK * 2;   // 16 KB of h
 constexpr uint32_t PT_B_STAGE = PT_BN * PT_BK * 2;   // 32 KB of W
 constexpr uint32_t PT_STAGE = PT_A_STAGE + PT_B_STAGE;
@@ -56,7 +58,8 @@ __global__ void __launch_bounds__(320, 1)
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int t0 = blockIdx.x * PT_BM, which = blockIdx.y, ks = blockIdx.z;
     const int kb = ks * kslice, ke = min(p.H, kb + kslice);
-    const int nch = (ke - kb + PT_BK - 1) / PT_BK;         // K-chunks of the slice, each taken twice (lo, hi)
+    const int nch = (ke - kb + PT_BK - 1) / PT_BK;         // K-chunks of the slice, each taken twice (hi and lo)
+    const bool paired = gridDim.x <= PT_PAIRED_TILES;      // lo first, two accumulators
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < PT_STAGES; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], 1); }
@@ -64,7 +67,7 @@ __global__ void __launch_bounds__(320, 1)
         sh.abort = 0;
         fence_barrier_init();
     }
-    if (warp == 1) { tmem_alloc(&sh.tmem_base, PT_NACC * PT_BN); tmem_relinquish(); }
+    if (warp == 1) { tmem_alloc(&sh.tmem_base, 2 * PT_BN); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -85,7 +88,7 @@ __global__ void __launch_bounds__(320, 1)
                 mbar_expect_tx(&sh.full[st], PT_STAGE);
                 const int kc = kb + (c % nch) * PT_BK;
                 tma_load_2d(sa, &tmap_h, &sh.full[st], kc, t0);
-                tma_load_2d(sa + PT_A_STAGE, c < nch ? &tmap_flo : &tmap_fhi, &sh.full[st], kc, which * RANK);
+                tma_load_2d(sa + PT_A_STAGE, (c < nch) == paired ? &tmap_flo : &tmap_fhi, &sh.full[st], kc, which * RANK);
                 pending |= 1u << st;
                 pend_par = (pend_par & ~(1u << st)) | (ph << st);
             }
@@ -102,10 +105,11 @@ __global__ void __launch_bounds__(320, 1)
                 if (!mbar_wait(&sh.full[st], (uint32_t)((c / PT_STAGES) & 1), abort)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t a0 = smem_u32(base + st * PT_STAGE), b0 = a0 + PT_A_STAGE;
+                const int acc = paired ? c % nch & 1 : 0;
 #pragma unroll
                 for (int kk = 0; kk < PT_BK / 16; ++kk)
-                    tc_mma_bf16(tmem + c % nch % PT_NACC * PT_BN, smem_desc_sw128(a0 + kk * 32),
-                                smem_desc_sw128(b0 + kk * 32), PT_IDESC, c >= PT_NACC || c >= nch || kk > 0);
+                    tc_mma_bf16(tmem + acc * PT_BN, smem_desc_sw128(a0 + kk * 32), smem_desc_sw128(b0 + kk * 32), PT_IDESC,
+                                c >= nch || c > acc || kk > 0);
                 tc_commit(&sh.empty[st]);
             }
             tc_commit(&sh.tfull);                  // also when stopped: the epilogue must not hang
@@ -124,7 +128,7 @@ __global__ void __launch_bounds__(320, 1)
             for (int c = 0; c < 4; ++c) {
                 float v[32];
                 tmem_ld32(tmem + lane_base + half * 128 + c * 32, v);
-                if (nch > 1) {
+                if (paired && nch > 1) {
                     float w[32];
                     tmem_ld32(tmem + lane_base + PT_BN + half * 128 + c * 32, w);
 #pragma unroll
@@ -146,7 +150,7 @@ __global__ void __launch_bounds__(320, 1)
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, PT_NACC * PT_BN);
+        tmem_dealloc(tmem, 2 * PT_BN);
     }
     if (threadIdx.x == 0 && sh.abort) set_status(p.status, ST_TIMEOUT);
 }
