@@ -203,3 +203,46 @@ def test_train_step_gradient_alignment(X):
         ref.train_step(*args, grads={**grads, "W_r": shifted(grads["W_r"])})
     assert err.value.code == X.XPRESS_ERR_INVALID_ARG
     ref.close()
+
+
+# A captured step: the work forked onto the refiner's own streams is part of the
+# graph, and a replay runs the whole step on what the inputs hold then (up to the
+# order of the atomic sums).
+def test_train_step_in_a_graph(X):
+    cfg = W.tiny_config("trgr", b=9, B=16, H=256, V=2088, r=256, dtype=W.BF16, seed=4600)
+    w = W.make_weights(cfg.H, cfg.V, cfg.r, cfg.B, cfg.dtype, 4601, "paper")
+    side = torch.cuda.Stream()
+    ref = X.Refiner({k: _bf16_dev(X, v) for k, v in w.items()}, cfg.H, cfg.V, cfg.r, cfg.B, X.XPRESS_BF16, stream=side)
+    names = ("h", "s", "target", "ystar", "anchor")
+
+    def inputs(seed):
+        inp = W.make_train_inputs(W.tiny_config("trgr", b=9, B=16, H=256, V=2088, r=256, dtype=W.BF16, seed=seed))
+        return [_bf16_dev(X, inp[k]) if k in names[:3] else torch.from_numpy(inp[k]).cuda() for k in names]
+
+    def eager(args):
+        torch.cuda.synchronize()
+        loss, grads = ref.train_step(*args)
+        torch.cuda.synchronize()
+        return loss, grads
+
+    args, other = inputs(4602), inputs(4603)
+    want = [eager(args), eager(other)]
+    loss, grads = torch.empty_like(want[0][0]), ref.alloc_grads()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        ref.train_step(*args, grads=grads, loss=loss)
+    for wl, wg in want:
+        for v in grads.values():
+            v.zero_()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert ref.device_status("train", cfg.b) == X.XPRESS_OK
+        np.testing.assert_array_equal(loss.cpu().numpy(), wl.cpu().numpy())
+        for k, v in wg.items():
+            np.testing.assert_allclose(grads[k].cpu().numpy(), v.cpu().numpy(), rtol=1e-5,
+                                       atol=1e-6 * float(v.abs().max()), err_msg=k)
+        for a, o in zip(args, other):
+            a.copy_(o)
+    ref.close()
