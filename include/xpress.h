@@ -167,7 +167,8 @@ int xpress_refine_block(const xpress_refiner *refiner, const xpress_block_in *in
                         void *stream);
 
 /* Acceptance of refined blocks against the target's logits (Sec. 3.1).
- *   target      [b, B+1, V] target logits for positions 1..B and the bonus
+ *   target      [b, B+1, V] target logits for positions 1..B and the bonus,
+ *               16-byte aligned
  *   s, tokens, lse, logit_sel, z_final: as passed to / returned by
  *               xpress_refine_block for the same blocks
  *   temperature [b] T <= 0: greedy -- accept the longest prefix equal to the
@@ -180,7 +181,8 @@ int xpress_refine_block(const xpress_refiner *refiner, const xpress_block_in *in
  * and s).
  * Outputs: accept_len [b] (0..B accepted draft tokens) and out_tokens
  * [b, B+1] (accepted tokens, then the correction or bonus token, then -1).
- * Errors: INVALID_ARG, WORKSPACE, CUDA. */
+ * Errors: INVALID_ARG (NULL pointer, target not 16-byte aligned, b < 1),
+ * WORKSPACE, CUDA. */
 typedef struct {
     int b;
     const void *target;

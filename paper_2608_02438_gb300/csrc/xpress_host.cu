@@ -1085,6 +1085,7 @@ int accept_launch(const xpress_refiner *R, const xpress_accept_in *in, int32_t *
     if (in->b < 1 || !in->target || !in->tokens || !in->temperature || !in->seed || !in->s || !in->lse ||
         !in->logit_sel || !in->z_final)
         return XPRESS_ERR_INVALID_ARG;
+    if (reinterpret_cast<uintptr_t>(in->target) & 15) return XPRESS_ERR_INVALID_ARG;   // read by 16-byte loads
     const AcceptLayout A = accept_layout(R, in->b);
     if (const int rc = check_ws(ws, ws_bytes, A.total)) return rc;
     char *w = static_cast<char *>(ws);

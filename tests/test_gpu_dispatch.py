@@ -283,3 +283,34 @@ def test_train_many_short_blocks(X):
     assert torch.allclose(loss, torch.cat(parts), rtol=1e-5, atol=1e-4)
     for k, g in grads.items():
         assert float((g - halves[k]).norm() / halves[k].norm()) < 6 * 2.0 ** -13, k
+
+
+def _at_offset(t, n):
+    """A copy of t whose first element lies n elements past an aligned address."""
+    flat = torch.empty(t.numel() + n, dtype=t.dtype, device="cuda")
+    flat[n:] = t.flatten()
+    return flat[n:].view(t.shape)
+
+
+# The acceptance reads the target's rows in 16-byte pieces: a target at another
+# boundary is refused, with and without a workspace.
+@pytest.mark.parametrize("dtype", [W.F32, W.BF16])
+def test_accept_refuses_an_unaligned_target(X, dtype):
+    cfg = W.tiny_config("acal", b=2, B=4, H=64, V=264, r=256, dtype=dtype, temps=(0.0, 1.0), seed=131)
+    inp = W.make_inputs(cfg)
+    ref, dt = _refiner(X, cfg, W.make_weights(cfg.H, cfg.V, cfg.r, cfg.B, cfg.dtype, 132, "paper"))
+    d = device_inputs(dt, inp)
+    o = ref.refine_block(d["h"], d["s"], d["draft"], d["anchor"], d["temperature"], d["seed"], inp["offset"], cfg.K_max)
+    out = dict(accept_len=torch.empty(2, dtype=torch.int32, device="cuda"),
+               out_tokens=torch.empty((2, 5), dtype=torch.int32, device="cuda"))
+    target = _at_offset(d["target"], 2)
+    with pytest.raises(X.XpressError) as err:
+        ref.accept(target, d["s"], o["tokens"], o["lse"], o["logit_sel"], o["z_final"], d["temperature"], d["seed"],
+                   inp["offset"], out=out)
+    assert err.value.code == X.XPRESS_ERR_INVALID_ARG
+    acc_in = X.XpressAcceptIn(2, *[t.data_ptr() for t in (target, d["s"], o["tokens"], o["lse"], o["logit_sel"],
+                                                          o["z_final"], d["temperature"], d["seed"])], inp["offset"])
+    with pytest.raises(X.XpressError) as err:
+        X.xpress_accept_noalloc(ref.handle, acc_in, out["accept_len"].data_ptr(), out["out_tokens"].data_ptr(),
+                                ref.stream.cuda_stream)
+    assert err.value.code == X.XPRESS_ERR_INVALID_ARG
