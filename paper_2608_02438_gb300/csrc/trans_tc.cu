@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(192, 1)
         if (got) {
             tc_fence_after();
             float *zf = p.z_final ? p.z_final : p.zbuf;
+            const bool zal = (reinterpret_cast<uintptr_t>(zf) & 15) == 0;   // the caller's z_final: any 4-byte boundary
 #pragma unroll
             for (int g = 0; g < TT_BN / 32; ++g) {
                 float v[32];
@@ -208,13 +209,20 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll
                     for (int c = 0; c < 4; ++c) dst[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
                 } else {
-                    float4 *zr = reinterpret_cast<float4 *>(zf + (size_t)tok * RANK + col);
+                    float *zr = zf + (size_t)tok * RANK + col;
                     uint32_t w[16];
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
                         const float4 x = cv[8 * g + c];
                         const float4 z = make_float4(x.x + v[4 * c], x.y + v[4 * c + 1], x.z + v[4 * c + 2], x.w + v[4 * c + 3]);
-                        zr[c] = z;
+                        if (zal) {
+                            reinterpret_cast<float4 *>(zr)[c] = z;
+                        } else {
+                            zr[4 * c] = z.x;
+                            zr[4 * c + 1] = z.y;
+                            zr[4 * c + 2] = z.z;
+                            zr[4 * c + 3] = z.w;
+                        }
                         w[2 * c] = (uint32_t)f2bf(z.x) | ((uint32_t)f2bf(z.y) << 16);
                         w[2 * c + 1] = (uint32_t)f2bf(z.z) | ((uint32_t)f2bf(z.w) << 16);
                     }

@@ -314,3 +314,21 @@ def test_accept_refuses_an_unaligned_target(X, dtype):
         X.xpress_accept_noalloc(ref.handle, acc_in, out["accept_len"].data_ptr(), out["out_tokens"].data_ptr(),
                                 ref.stream.cuda_stream)
     assert err.value.code == X.XPRESS_ERR_INVALID_ARG
+
+
+# z_final at a 4-byte boundary, on each path that writes it: fp32, the persistent
+# kernel, and the token tiles of k_trans_tc.
+@pytest.mark.parametrize("dtype,b,B", [(W.F32, 3, 5), (W.BF16, 2, 16), (W.BF16, 9, 15)])
+def test_z_final_at_any_boundary(X, dtype, b, B):
+    cfg = W.tiny_config("zal", b=b, B=B, H=64, V=2056, r=256, dtype=dtype, temps=(0.0, 1.0), seed=141)
+    inp = W.make_inputs(cfg)
+    ref, dt = _refiner(X, cfg, W.make_weights(cfg.H, cfg.V, cfg.r, cfg.B, cfg.dtype, 142, "strong"))
+    d = device_inputs(dt, inp)
+    args = (d["h"], d["s"], d["draft"], d["anchor"], d["temperature"], d["seed"], inp["offset"], cfg.K_max)
+    want = ref.refine_block(*args)
+    got = ref.alloc_outputs(b)
+    got["z_final"] = _at_offset(torch.full_like(got["z_final"], float("nan")), 1)
+    ref.refine_block(*args, out=got)
+    torch.cuda.synchronize()
+    assert ref.device_status("refine", b) == X.XPRESS_OK
+    assert torch.equal(got["z_final"], want["z_final"]) and torch.equal(got["tokens"], want["tokens"])
