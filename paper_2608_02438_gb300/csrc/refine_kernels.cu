@@ -353,7 +353,12 @@ __global__ void __launch_bounds__(256) k_pre_mix(const Params *__restrict__ pp)
         float *ug = U + B * 2 * RANK;          // [r]       W_g g
         float *Ws = ug + RANK;                 // [32][2r + 4]  W_in[d0 + dd][0:2r] (8 rows' 16-byte reads meet 8 bank groups)
         P = Ws + 32 * WS_LD;
-        if (p.dtype) {
+        if (p.dtype && !al16(p.W_in)) {        // W_in at a 2-byte boundary
+            const uint16_t *W = static_cast<const uint16_t *>(p.W_in);
+#pragma unroll 8
+            for (int i = threadIdx.x; i < 32 * 2 * RANK; i += 256)
+                Ws[i / (2 * RANK) * WS_LD + i % (2 * RANK)] = bf2f(W[(size_t)(d0 + i / (2 * RANK)) * 3 * RANK + i % (2 * RANK)]);
+        } else if (p.dtype) {
             constexpr int PER = 32 * 2 * RANK / 8 / 256;   // 8 16-byte pieces per thread
             uint4 wv[PER];
 #pragma unroll

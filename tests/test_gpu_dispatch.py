@@ -332,3 +332,24 @@ def test_z_final_at_any_boundary(X, dtype, b, B):
     torch.cuda.synchronize()
     assert ref.device_status("refine", b) == X.XPRESS_OK
     assert torch.equal(got["z_final"], want["z_final"]) and torch.equal(got["tokens"], want["tokens"])
+
+
+# W_in of a bf16 refiner at a 2-byte boundary: the precompute that folds it in per
+# call (at most 32 tokens, H not a multiple of 64), and those that take the
+# refiner's folded copy.
+@pytest.mark.parametrize("b,B,H", [(2, 8, 72), (2, 8, 128), (5, 16, 128)])
+def test_bf16_W_in_at_any_boundary(X, b, B, H):
+    cfg = W.tiny_config("wal", b=b, B=B, H=H, V=2056, r=256, dtype=W.BF16, temps=(0.0, 1.0), seed=151)
+    inp = W.make_inputs(cfg)
+    w = {k: X.to_device(v, X.XPRESS_BF16)
+         for k, v in W.make_weights(cfg.H, cfg.V, cfg.r, cfg.B, cfg.dtype, 152, "strong").items()}
+    d = device_inputs(X.XPRESS_BF16, inp)
+    outs = []
+    for weights in (w, {**w, "W_in": _at_offset(w["W_in"], 1)}):
+        ref = X.Refiner(weights, cfg.H, cfg.V, cfg.r, cfg.B, X.XPRESS_BF16)
+        outs.append(ref.refine_block(d["h"], d["s"], d["draft"], d["anchor"], d["temperature"], d["seed"],
+                                     inp["offset"], cfg.K_max))
+        torch.cuda.synchronize()
+        assert ref.device_status("refine", b) == X.XPRESS_OK
+    for k in ("tokens", "iters", "z_final", "logit_sel"):
+        assert torch.equal(outs[0][k], outs[1][k]), k
