@@ -412,28 +412,14 @@ namespace {
 constexpr int DRAW_NZ = 16;         // fp32: draws per sweep of the vocabulary (accumulators per lane)
 constexpr int DRAW_THREADS = 256;
 
-// 32 consecutive elements of row v of W_r (bf16 or fp32) as floats.
-__device__ __forceinline__ void load_row32(float (&w)[32], const void *W_r, int dtype, int v, int k0)
+// 32 consecutive elements of row v of the fp32 W_r.
+__device__ __forceinline__ void load_row32(float (&w)[32], const void *W_r, bool al, int v, int k0)
 {
-    if (dtype) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(W_r) + (size_t)v * RANK + k0);
+    const float *src = static_cast<const float *>(W_r) + (size_t)v * RANK + k0;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const uint4 x = __ldg(src + c);
-            const uint32_t ww[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                w[8 * c + 2 * q] = __uint_as_float(ww[q] << 16);
-                w[8 * c + 2 * q + 1] = __uint_as_float(ww[q] & 0xFFFF0000u);
-            }
-        }
-    } else {
-        const float4 *src = reinterpret_cast<const float4 *>(static_cast<const float *>(W_r) + (size_t)v * RANK + k0);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const float4 x = __ldg(src + c);
-            w[4 * c] = x.x; w[4 * c + 1] = x.y; w[4 * c + 2] = x.z; w[4 * c + 3] = x.w;
-        }
+    for (int c = 0; c < 8; ++c) {
+        const float4 x = ld4(src + 4 * c, al);
+        w[4 * c] = x.x; w[4 * c + 1] = x.y; w[4 * c + 2] = x.z; w[4 * c + 3] = x.w;
     }
 }
 }  // namespace
@@ -518,6 +504,7 @@ __global__ void __launch_bounds__(DRAW_THREADS) k_acc_draw_simt(AcceptParams p)
     __shared__ DrawDesc dsc[DRAW_NZ];
     __shared__ unsigned long long wkey[DRAW_THREADS / 32][DRAW_NZ][2];
     __shared__ int s_any_resid, s_last;
+    const bool wal = al16(p.W_r);
     for (int g0 = 0; g0 < nd; g0 += DRAW_NZ) {
         const int nz = min(DRAW_NZ, nd - g0);
         if (threadIdx.x < nz) dsc[threadIdx.x] = list[g0 + threadIdx.x];
@@ -546,7 +533,7 @@ __global__ void __launch_bounds__(DRAW_THREADS) k_acc_draw_simt(AcceptParams p)
 #pragma unroll 1
                 for (int k0 = 0; k0 < RANK; k0 += 32) {
                     float w[32];
-                    load_row32(w, p.W_r, p.dtype, v, k0);
+                    load_row32(w, p.W_r, wal, v, k0);
 #pragma unroll
                     for (int j = 0; j < DRAW_NZ; ++j) {
                         if (j < nz) {

@@ -555,6 +555,15 @@ __device__ __forceinline__ void select_group_warp(SelState &st, const float (&l)
     }
 }
 
+// Four consecutive floats, as one 16-byte load where the array allows it
+// (fp32 weights may sit at any 4-byte boundary).
+__device__ __forceinline__ float4 ld4(const float *q, bool al)
+{
+    if (al) return __ldg(reinterpret_cast<const float4 *>(q));
+    return make_float4(__ldg(q), __ldg(q + 1), __ldg(q + 2), __ldg(q + 3));
+}
+__device__ __forceinline__ bool al16(const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; }
+
 // ------------------------------------------------------------- PTX wrappers
 
 __device__ __forceinline__ unsigned long long globaltimer_ns()

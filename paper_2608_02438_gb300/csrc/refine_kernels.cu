@@ -176,14 +176,6 @@ __device__ __forceinline__ void gemm_nt_tile(const TA *__restrict__ A, int lda, 
         }
 }
 
-// Four consecutive floats, as one 16-byte load where the array allows it
-// (fp32 weights may sit at any 4-byte boundary).
-__device__ __forceinline__ float4 ld4(const float *q, bool al)
-{
-    if (al) return __ldg(reinterpret_cast<const float4 *>(q));
-    return make_float4(__ldg(q), __ldg(q + 1), __ldg(q + 2), __ldg(q + 3));
-}
-__device__ __forceinline__ bool al16(const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; }
 __device__ __forceinline__ float dot4(const float4 &a, const float4 &b, float c)
 {
     return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));

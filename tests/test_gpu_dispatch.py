@@ -353,3 +353,24 @@ def test_bf16_W_in_at_any_boundary(X, b, B, H):
         assert ref.device_status("refine", b) == X.XPRESS_OK
     for k in ("tokens", "iters", "z_final", "logit_sel"):
         assert torch.equal(outs[0][k], outs[1][k]), k
+
+
+# The fp32 residual draw with W_r at a 4-byte boundary.
+def test_fp32_draw_with_W_r_at_any_boundary(X):
+    cfg = W.tiny_config("wral", b=5, B=4, H=64, V=1032, r=256, dtype=W.F32, temps=(1.0, 0.7), seed=161,
+                        logits="gauss4_spike", draft="sample")
+    inp = W.make_inputs(cfg)
+    w = {k: X.to_device(v, X.XPRESS_F32)
+         for k, v in W.make_weights(cfg.H, cfg.V, cfg.r, cfg.B, cfg.dtype, 162, "strong").items()}
+    d = device_inputs(X.XPRESS_F32, inp)
+    outs = []
+    for weights in (w, {**w, "W_r": _at_offset(w["W_r"], 1)}):
+        ref = X.Refiner(weights, cfg.H, cfg.V, cfg.r, cfg.B, X.XPRESS_F32)
+        o = ref.refine_block(d["h"], d["s"], d["draft"], d["anchor"], d["temperature"], d["seed"], inp["offset"], cfg.K_max)
+        outs.append(ref.accept(d["target"], d["s"], o["tokens"], o["lse"], o["logit_sel"], o["z_final"],
+                               d["temperature"], d["seed"], inp["offset"]))
+        torch.cuda.synchronize()
+        assert ref.device_status("accept", cfg.b) == X.XPRESS_OK
+    assert int(outs[0]["accept_len"].min()) < cfg.B                # at least one residual draw
+    for k in ("accept_len", "out_tokens"):
+        assert torch.equal(outs[0][k], outs[1][k]), k
