@@ -446,16 +446,6 @@ __device__ __forceinline__ void draw_finish(const AcceptParams &p, const DrawDes
     }
 }
 
-// The Gumbel noise of ids v and v + 1 (v even: one Philox call gives both).
-__device__ __forceinline__ void gumbel_pair(unsigned long long seed, uint32_t v, uint32_t pos, uint32_t stream,
-                                            uint32_t offset, float &g0, float &g1)
-{
-    const uint4 o = philox10(make_uint4(v >> 2, pos, stream, offset), (uint32_t)seed, (uint32_t)(seed >> 32));
-    const uint32_t w0 = (v & 2u) ? o.z : o.x, w1 = (v & 2u) ? o.w : o.y;
-    g0 = -logf(-logf(((float)(w0 >> 9) + 0.5f) * (1.0f / 8388608.0f)));
-    g1 = -logf(-logf(((float)(w1 >> 9) + 0.5f) * (1.0f / 8388608.0f)));
-}
-
 // Scores of one (draw, vocabulary id) pair, merged into the lane's running
 // bests: the p draw tx + g, and for a residual draw log(max(0, p - q)) + g
 // with l = acc + s recomputed (acc = (W_r z)_v).

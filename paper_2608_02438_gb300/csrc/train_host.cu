@@ -329,9 +329,9 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
     tp.status = m.status;
     tp.wait_ns = refiner_wait_ns(R);
 
-    CUtensorMap tz128, tz64, tw64, tw128, ts64, tt64, tg;
-    if (!tmap_bf16(&tz128, U(L.zop), r, NR, r, 64, 128) || !tmap_bf16_kblocks(&tz64, U(L.zop), NR, 64) ||
-        !tmap_bf16_kblocks(&tw64, w.W_r, V, 64) || !tmap_bf16_kblocks(&tw128, w.W_r, V, 128) ||
+    CUtensorMap tz64, tw64, tw128, ts64, tt64, tg;
+    if (!tmap_bf16_kblocks(&tz64, U(L.zop), NR, 64) || !tmap_bf16_kblocks(&tw64, w.W_r, V, 64) ||
+        !tmap_bf16_kblocks(&tw128, w.W_r, V, 128) ||
         !tmap_bf16(&ts64, in->s, V, P, V, 64, 64) || !tmap_bf16(&tt64, in->target, V, P, V, 64, 64) ||
         !tmap_f32_rank(&tg, out->gW_r, V))
         return XPRESS_ERR_CUDA;
@@ -342,7 +342,7 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
     auto run_dz = [&](int j0, int n) {
         TrainParams q = tp;
         q.j0 = j0;
-        return launch(k_train_tok_dz, dim3(L.splits, n), dim3(kTrainTokThreads), kTrainTokSmemBytes, st, q, tz128, tw64,
+        return launch(k_train_tok_dz, dim3(L.splits, n), dim3(kTrainTokThreads), kTrainTokSmemBytes, st, q, tw64,
                       ts64, tt64);
     };
     auto run_dw = [&](int j0, int n, cudaStream_t s, int ctas) {
@@ -353,10 +353,10 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
     };
     if (only >= 0) {
         if (only == TR_STATS)
-            XT_CUDA(launch(k_train_tok_stats, gtok, dim3(kTrainTokThreads), kTrainTokSmemBytes, st, tp, tz128,
+            XT_CUDA(launch(k_train_tok_stats, gtok, dim3(kTrainTokThreads), kTrainTokSmemBytes, st, tp,
                            tw128, ts64, tt64));
         else if (only == TR_TV)
-            XT_CUDA(launch(k_train_tok_tv, gtok, dim3(kTrainTokThreads), kTrainTokSmemBytes, st, tp, tz128, tw64, ts64,
+            XT_CUDA(launch(k_train_tok_tv, gtok, dim3(kTrainTokThreads), kTrainTokSmemBytes, st, tp, tw64, ts64,
                            tt64));
         else
             for (int j0 = 0; j0 < mt; j0 += L.dl_tiles) {
@@ -403,10 +403,10 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
 
     // the Read passes
     // W_r tiles of 128 ids (boxes of 128 rows) for the log-sum-exp pass, of 64 for the others
-    XT_CUDA(launch(k_train_tok_stats, gtok, dim3(kTrainTokThreads), kTrainTokSmemBytes, st, tp, tz128, tw128,
+    XT_CUDA(launch(k_train_tok_stats, gtok, dim3(kTrainTokThreads), kTrainTokSmemBytes, st, tp, tw128,
                    ts64, tt64));
     XT_CUDA(launch(k_train_stats_fin, dim3(NR / 8), dim3(256), 0, st, m));
-    XT_CUDA(launch(k_train_tok_tv, gtok, dim3(kTrainTokThreads), kTrainTokSmemBytes, st, tp, tz128, tw64, ts64,
+    XT_CUDA(launch(k_train_tok_tv, gtok, dim3(kTrainTokThreads), kTrainTokSmemBytes, st, tp, tw64, ts64,
                    tt64));
     XT_CUDA(launch(k_train_tv_fin, dim3(in->b), dim3(32, in->B), 0, st, m));
     // The refiner's own streams beside `st`: one for the dL/dW_r product, one for

@@ -522,14 +522,13 @@ __global__ void __launch_bounds__(1024) k_train_tv_fin(TrainMisc m)
     const int blk = blockIdx.x, k = threadIdx.y, lane = threadIdx.x;
     const int i = blk * m.B + k;
     __shared__ float sl[3][MAX_B];
-    float sum[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}}, anc = 0.f;   // per forward: x, y, z of the partials
+    float sum[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, anc = 0.f;   // per forward: x, y of the partials
     for (int sv = lane; sv < m.splits; sv += 32) {
 #pragma unroll
         for (int f = 0; f < 2; ++f) {
             const float4 a = m.part[(size_t)sv * m.NR + pair_row(i, f)];
             sum[f][0] += a.x;
             sum[f][1] += a.y;
-            sum[f][2] += a.z;
             anc += a.w;
         }
     }
@@ -538,7 +537,7 @@ __global__ void __launch_bounds__(1024) k_train_tv_fin(TrainMisc m)
 #pragma unroll
         for (int f = 0; f < 2; ++f)
 #pragma unroll
-            for (int q = 0; q < 3; ++q) sum[f][q] += __shfl_xor_sync(0xffffffffu, sum[f][q], o);
+            for (int q = 0; q < 2; ++q) sum[f][q] += __shfl_xor_sync(0xffffffffu, sum[f][q], o);
         anc += __shfl_xor_sync(0xffffffffu, anc, o);
     }
     if (lane == 0) {
@@ -546,10 +545,10 @@ __global__ void __launch_bounds__(1024) k_train_tv_fin(TrainMisc m)
         float lf[2];
         for (int f = 0; f < 2; ++f) {
             const int row = pair_row(i, f);
-            const float sm = sum[f][0], lt = sum[f][1], eq = sum[f][2];
+            const float sm = sum[f][0], lt = sum[f][1];
             // lt: sum of p where p < q plus half of it where p = q (k_train_tok)
             const float l1 = 2.0f * (1.0f - sm);
-            const float S = 1.0f - 2.0f * lt - eq;          // sum_v sgn(p_v - q_v) p_v
+            const float S = 1.0f - 2.0f * lt;               // sum_v sgn(p_v - q_v) p_v
             const float ce = m.lse_p2[row] * LN2 - m.ly[row];
             lf[f] = w * (m.a_ce * ce + m.a_l1 * l1);
             // dL/dl_v = cf [a_ce (p_v - [v = y*]) + a_l1 p_v (sgn(p_v - q_v) - S)]

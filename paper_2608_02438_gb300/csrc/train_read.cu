@@ -623,26 +623,22 @@ __device__ __forceinline__ void train_tok_body(const TrainParams &p, const CUten
     if (threadIdx.x == 0 && sh.abort) set_status(p.status, ST_TIMEOUT);
 }
 
-// grid (splits, row tiles from p.j0 on), TR_THREADS threads, TR_SMEM bytes; one kernel per
-// mode.  tmap_z is not read (Z goes to tensor memory from p.zop).
+// grid (splits, row tiles from p.j0 on), TR_THREADS threads, TR_SMEM bytes; one kernel per mode.
 __global__ void __launch_bounds__(TR_THREADS, 1)
-    k_train_tok_stats(const __grid_constant__ TrainParams p, const __grid_constant__ CUtensorMap tmap_z,
-                      const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_s,
-                      const __grid_constant__ CUtensorMap tmap_t)
+    k_train_tok_stats(const __grid_constant__ TrainParams p, const __grid_constant__ CUtensorMap tmap_w,
+                      const __grid_constant__ CUtensorMap tmap_s, const __grid_constant__ CUtensorMap tmap_t)
 {
     train_tok_body<TR_STATS>(p, tmap_w, tmap_s, tmap_t);
 }
 __global__ void __launch_bounds__(TR_THREADS, 1)
-    k_train_tok_tv(const __grid_constant__ TrainParams p, const __grid_constant__ CUtensorMap tmap_z,
-                   const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_s,
-                   const __grid_constant__ CUtensorMap tmap_t)
+    k_train_tok_tv(const __grid_constant__ TrainParams p, const __grid_constant__ CUtensorMap tmap_w,
+                   const __grid_constant__ CUtensorMap tmap_s, const __grid_constant__ CUtensorMap tmap_t)
 {
     train_tok_body<TR_TV>(p, tmap_w, tmap_s, tmap_t);
 }
 __global__ void __launch_bounds__(TR_THREADS, 1)
-    k_train_tok_dz(const __grid_constant__ TrainParams p, const __grid_constant__ CUtensorMap tmap_z,
-                   const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_s,
-                   const __grid_constant__ CUtensorMap tmap_t)
+    k_train_tok_dz(const __grid_constant__ TrainParams p, const __grid_constant__ CUtensorMap tmap_w,
+                   const __grid_constant__ CUtensorMap tmap_s, const __grid_constant__ CUtensorMap tmap_t)
 {
     train_tok_body<TR_DZ>(p, tmap_w, tmap_s, tmap_t);
 }
