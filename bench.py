@@ -49,7 +49,7 @@ SMALL_SOURCES = [CSRC + f for f in ("refine_small.cu", "tcv_common.cuh", "mlp_co
 SMALL_SUMMARY = "profiles/k_refine_small_qwen3_8b_greedy.txt"
 READ_SOURCES = [CSRC + "read_tc.cu", CSRC + "common.cuh"]
 READ_SUMMARIES = {"long_b64": "profiles/k_read_tc_long_b64.txt"}
-LM_SOURCES = [CSRC + "lm_head.cu", CSRC + "common.cuh"]
+LM_SOURCES = [CSRC + "lm_head.cu", CSRC + "lm_work.h", CSRC + "common.cuh"]
 TRAIN_SOURCES = [CSRC + f for f in ("train_read.cu", "train_common.cuh", "kernels.h", "common.cuh")]
 TRAIN_SUMMARIES = {"dz": "profiles/k_train_tok_dz_qwen3_8b_train.txt", "dW_r": "profiles/k_train_dw_qwen3_8b_train.txt"}
 LM_SUMMARIES = {16: "profiles/k_lm_head32_qwen3_8b_n16.txt"}
@@ -252,15 +252,23 @@ def run_reference(args):
     return 0
 
 
-def lm_head_line(us, nbytes, flops, hbm, tc_peak, tokens):
+def lm_head_kernel(V, tokens, sms):
+    """The LM head kernel that the library takes for these sizes (lm_shape in
+    xpress_host.cu)."""
+    if tokens <= 128:
+        return "k_lm_head32" if tokens <= 32 else "k_lm_head128"
+    ctas = min(-(-V // 128), sms)
+    return "k_lm_head256x2" if -(-tokens // 256) * -(-V // 256) >= 2 * ctas else "k_lm_head256"
+
+
+def lm_head_line(us, nbytes, flops, hbm, tc_peak, tokens, V, sms):
     """The base-logit LM head against its roofline: the weight stream (HBM)
     for few tokens, the bf16 tensor pipe once the arithmetic intensity nears
     the ridge point."""
     gbs = nbytes / (us * 1e-6) / 1e9
     tfs = flops / (us * 1e-6) / 1e12
     tensor = flops / nbytes >= 0.75 * tc_peak * 1e3 / hbm
-    kernel = "k_lm_head32" if tokens <= 32 else "k_lm_head128" if tokens <= 128 else "k_lm_head256x2"
-    return {"kernel": kernel, "us_per_call": us, "tokens": tokens,
+    return {"kernel": lm_head_kernel(V, tokens, sms), "us_per_call": us, "tokens": tokens,
             "bytes_per_call": nbytes, "flops_per_call": flops, "achieved_gbs": gbs, "achieved_tflops": tfs,
             "bound": "tensor" if tensor else "hbm", "peak": tc_peak if tensor else hbm,
             "frac": tfs / tc_peak if tensor else gbs / hbm,
@@ -630,7 +638,8 @@ def run_xpress(args):
             "sequential_decode_us_per_call": seq_us,
             "markov_head_us_per_call": markov_us,
             "lm_head": None if lm_us is None else dict(
-                lm_head_line(lm_us, lm_bytes, 2.0 * cfg.V * cfg.H * b * cfg.B, hbm, tc_peak, b * cfg.B),
+                lm_head_line(lm_us, lm_bytes, 2.0 * cfg.V * cfg.H * b * cfg.B, hbm, tc_peak, b * cfg.B, cfg.V,
+                             torch.cuda.get_device_properties(dev).multi_processor_count),
                 traffic=profiled_traffic(LM_SUMMARIES.get(b * cfg.B, ""), source_hash(LM_SOURCES))),
             "train_step": train,
             "e2e": {"value": e2e_value, "unit": "blocks/s", "h2d_bytes_per_step": int(h2d),

@@ -61,3 +61,11 @@ def test_committed_summaries_name_their_kernel_sources(bench):
                 kv[k.strip()] = v.strip()
         assert len(kv.get("source_hash", "")) == 16, rel
         assert float(kv["dram_bytes_per_launch"]) > 0, rel
+
+
+@pytest.mark.parametrize("V,tokens,kernel", [(151936, 16, "k_lm_head32"), (151936, 33, "k_lm_head128"),
+                                             (151936, 129, "k_lm_head256x2"), (77824, 129, "k_lm_head256x2"),
+                                             (77568, 256, "k_lm_head256"), (2088, 512, "k_lm_head256"),
+                                             (2088, 1025, "k_lm_head256x2")])
+def test_lm_head_kernel_is_the_one_launched(bench, V, tokens, kernel):
+    assert bench.lm_head_kernel(V, tokens, 152) == kernel
