@@ -166,18 +166,19 @@ struct RowState {
 // waits for that kernel before it exits, so that the later kernels' waits
 // cover it too.  It clears the status word and the draw counters.
 //
-// Bound by the target's stream from HBM.  The pieces of a thread's next batch
-// (four of 16
-// bytes, of the next item once the current one is used up) are
-// requested before the current batch is reduced, so the loads never stop for the
-// arithmetic or for an item's merge, which costs five shuffle rounds and one
-// barrier (double-buffered by item parity).  bf16 maxima are taken on the packed
-// words and the exponentials' arguments and sums in packed fp32.  Measured under
-// ncu at 2112 rows of 151936 bf16, half of them sampling: 219 us with the loads of
-// a batch issued after the previous batch's arithmetic and a shared-memory tree
-// per item, 153 with batches ahead, 144 with the packed arithmetic (4.5 TB/s);
-// 544 sampling rows 66, 46, 43.  Eight pieces and 3 CTAs an SM took 138 and 43 and
-// made a call of one block 1 % slower; other cache hints change nothing.
+// The pieces of a thread's next batch (four of 16 bytes, of the next item once the
+// current one is used up) are requested before the current batch is reduced, so
+// the loads do not wait for the arithmetic or for an item's merge, which costs five
+// shuffle rounds and one barrier (double-buffered by item parity).  bf16 maxima are
+// taken on the packed words and the exponentials' arguments and sums in packed
+// fp32.  Measured under ncu at 2112 rows of 151936 bf16, half of them sampling: 219
+// us with the loads of a batch issued after the previous batch's arithmetic and a
+// shared-memory tree per item, 153 with batches ahead, 144 with the packed
+// arithmetic; 544 sampling rows 66, 46, 43.  That is 4.5 and 3.8 TB/s, 0.67 and 0.58
+// of the copy bandwidth, so HBM alone does not bound it: what is left is the mix of
+// the exponentials' issue slots and of the bytes that registers hold in flight.
+// Eight pieces and 3 CTAs an SM took 138 and 43 and made a call of one block 1 %
+// slower; other cache hints change nothing.
 namespace {
 
 constexpr int ROWS_U = 4;                         // pieces in flight per thread and batch

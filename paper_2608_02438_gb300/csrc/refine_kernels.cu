@@ -70,13 +70,13 @@ __global__ void k_init(Params pin, Params *pdev, cudaGraphConditionalHandle hand
 // --------------------------------------------------------------- k_rowmax
 
 // One CTA per row: first index of the maximum of s[row, :] (fp32 compare).
-// grid N, 1024 threads.  HBM-bound over s: 16-byte pieces (V % 8 == 0 and an
-// aligned s make every piece whole), four in flight per thread, so that a CTA
-// keeps 64 KB in flight and even the 33 rows of the smallest batch that comes
-// here fill the memory system.  Each thread meets its ids in increasing order
-// and keeps the first maximum; the merges keep the smaller id.  Measured at
-// 80 rows of 151936 bf16: a whole round 222 us against 481 us with 2-byte loads in
-// 256 threads (271 us of it this kernel, now about 12).
+// grid N, 1024 threads: 16-byte pieces (V % 8 == 0 and an aligned s make every piece
+// whole), four in flight per thread, so that a CTA keeps 64 KB in flight (bf16
+// refiners come here with 33 rows or more, fp32 ones with any number, and with
+// fewer rows than SMs the other SMs stay idle).  Each thread meets its ids in
+// increasing order and keeps the first maximum; the merges keep the smaller id.
+// Measured at 80 rows of 151936 bf16: a whole round 222 us against 481 us with 2-byte
+// loads in 256 threads (271 us of it this kernel, now about 12: 24 MB at 2 TB/s).
 template <int DT>
 __device__ __forceinline__ void rowmax_scan(const Params &p, size_t row, float &best, int &idx)
 {

@@ -26,10 +26,13 @@ namespace {
         }                                                                                                      \
     } while (0)
 
-// SMs that the dL/dW_r product leaves to the backward chain beside it: a step of
-// 32 blocks of 16 took 762 us with the product before the chain, 746 with 24
-// SMs left, 732 with 32, 726 with 56 (its 96 CTAs still draw the HBM rate); one of
-// 6 blocks at V = 32008 203, 192, 192, 191.
+// SMs that the dL/dW_r product leaves to the backward chain beside it.  A step with
+// the product before the chain / beside it with 0, 24, 56 SMs left, us: 512
+// positions 685 / 673, 667, 647 (the product's 96 CTAs still draw the HBM rate
+// there), 1024 1804 / 1791, 1769, 1770, 2048 3416 / 3404, 3400, 3395, 4096 4684 /
+// 4671, 4655, 4661, 12800 17237 / 17222, 17217, 17205 (V = 151936); 4096 at V = 32008
+// 1351 / 1330, 1325, 1337.  With more positions the product is as long on fewer SMs
+// as the chain is short, and the number matters less.
 constexpr int TRAIN_DW_LEAVE = 56;
 
 size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -425,8 +428,7 @@ int train_run(const xpress_refiner *R, const xpress_train_in *in, const xpress_t
         // The last (mostly the only) group's dL/dW_r product runs on a stream of
         // its own beside the backward chain below, which is a row of small,
         // latency-bound kernels: TRAIN_DW_LEAVE SMs stay free for their products
-        // (the others' shared memory is taken), and the HBM-bound product does
-        // not need them.  Both add into gW_r atomically.
+        // (the others' shared memory is taken).  Both add into gW_r atomically.
         XT_CUDA(dw_fork.fork(ev[4]));
         XT_CUDA(run_dw(j0, n, dw_stream, sms > 2 * TRAIN_DW_LEAVE ? sms - TRAIN_DW_LEAVE : sms));
     }

@@ -207,8 +207,9 @@ Layout make_layout(const xpress_refiner *R, int b)
         L.ksplit = (R->w.H + L.kchunk - 1) / L.kchunk;
     } else if (R->use_tc) {
         // k_pre_tc: 128-token x 256-row tiles, split over K to about one wave, at
-        // most PRE_TC_SPLITS ways (k_pre_mix adds every split of an element: at 80
-        // tokens 64 splits took 28 us for the two kernels, 16 take 22)
+        // most PRE_TC_SPLITS ways, since k_pre_mix adds every split of an element: a
+        // call of one pass takes, with one wave's splits / 16, 64.5 / 57.7 us at 48
+        // tokens, 68.0 / 61.5 at 80, 69.8 / 66.1 at 144 and 73.8 / 73.2 at 320
         L.pre_tc = true;
         const int tiles = 2 * ((N + 127) / 128);
         int ks = (R->num_sms + tiles / 2) / tiles;
@@ -1223,8 +1224,8 @@ int lm_grid(int V)
 }
 
 // The kernel for N tokens of a V-row head on G CTAs: the narrowest token chunk
-// that holds them all, else 256 tokens, by two vocabulary tiles where every CTA
-// still gets two items (lm_head.cu has both sides' times).
+// that holds them all, else 256 tokens, by two vocabulary tiles where there are
+// still two such items for each CTA (lm_head.cu has both sides' times).
 const LmKernel &lm_shape(int V, int N, int G)
 {
     if (N <= 32) return kLmHeads[0];
