@@ -160,7 +160,9 @@ size_t xpress_refine_workspace_size(const xpress_refiner *refiner, int b);
  * pass re-evaluates only the positions after the first token the previous
  * pass changed (by Theorem 1 the others cannot change).  workspace: >= the
  * size above, 256-byte aligned, owned by the caller, not shared by concurrent
- * calls.
+ * calls and not written by anything but this function while the refiner uses it
+ * (the small-batch kernel keeps its hand-off counters there from call to call, so
+ * the same bytes do not serve as another call's workspace in between).
  * Errors: INVALID_ARG, UNSUPPORTED, WORKSPACE, CUDA. */
 int xpress_refine_block(const xpress_refiner *refiner, const xpress_block_in *in,
                         const xpress_block_out *out, void *workspace, size_t ws_bytes,

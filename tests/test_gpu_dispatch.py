@@ -374,3 +374,10 @@ def test_fp32_draw_with_W_r_at_any_boundary(X):
     assert int(outs[0]["accept_len"].min()) < cfg.B                # at least one residual draw
     for k in ("accept_len", "out_tokens"):
         assert torch.equal(outs[0][k], outs[1][k]), k
+
+
+# Draws of more than two sweeps of the vocabulary: 87 in three of 32 (bf16), 40 in
+# three of 16 (fp32).
+@pytest.mark.parametrize("b,V,dtype", [(130, 264, W.BF16), (60, 296, W.F32)])
+def test_accept_many_sweeps(X, b, V, dtype):
+    test_accept_row_and_draw_edges(X, b, V, dtype, 0)
